@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <cstdio>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/life.h"
@@ -38,7 +39,8 @@ struct Err {
 #define LIFE_CHECK_LAUNCH() LIFE_CUDA_TRY(cudaGetLastError())
 
 // Device-side status word (bounded waits record a timeout here, never trap).
-enum : uint32_t { DEV_OK = 0, DEV_TIMEOUT = 1u, DEV_BAD_INDEX = 2u, DEV_BAD_VALUE = 4u };
+enum : uint32_t { DEV_OK = 0, DEV_TIMEOUT = 1u, DEV_BAD_INDEX = 2u, DEV_BAD_VALUE = 4u,
+                DEV_UNSORTED = 8u };  // DEV_UNSORTED: the fascicle ids of a raw list are not in order
 // Device word that bounded waits set (per device, allocated on first use).
 uint32_t* dev_status_word();
 
@@ -92,6 +94,10 @@ struct TmpBuf {
             return LIFE_ENOMEM;
         }
         return LIFE_OK;
+    }
+    void swap(TmpBuf& o) {
+        std::swap(p, o.p);
+        std::swap(s, o.s);
     }
     template <class T> T* as() const { return static_cast<T*>(p); }
 };
@@ -263,7 +269,7 @@ life_status export_layout(life_index_s* ix, int layout, int32_t* atom, int32_t* 
                           float* val, cudaStream_t s);
 
 // Sorting and scans (index_build.cu)
-life_status radix_sort_pairs(uint64_t* keys, uint32_t* vals, int64_t n, int bits, cudaStream_t s);
+life_status radix_sort_pairs(TmpBuf& keys, TmpBuf& vals, int64_t n, int bit0, int bit1, cudaStream_t s);
 life_status exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t n, cudaStream_t s);
 
 // ------------------------------------------------------------ SIMT SpMVs

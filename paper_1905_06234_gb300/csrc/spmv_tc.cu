@@ -697,11 +697,12 @@ life_status build_tile_layout(life_index_s* ix, cudaStream_t s) {
                                                       (1ull << bf) - 1, bf, d_vox_tile.as<int32_t>(),
                                                       d_vox_row.as<int32_t>(), skey.as<uint64_t>(), spay.as<uint32_t>());
             LIFE_CHECK_LAUNCH();
-            LIFE_TRY(radix_sort_pairs(skey.as<uint64_t>(), spay.as<uint32_t>(), m, bt + 16 + bf, s));
+            // from (v, a, f) order by a stable sort: a cell's entries keep their fascicle order
+            LIFE_TRY(radix_sort_pairs(skey, spay, m, bf, bt + 16 + bf, s));
             brick_key_kernel<<<grid1d(m), 256, 0, s>>>(skey.as<uint64_t>(), m, bf, d_tile_brick.as<int32_t>(),
                                                        key2.as<uint64_t>(), pay2.as<uint32_t>());
             LIFE_CHECK_LAUNCH();
-            LIFE_TRY(radix_sort_pairs(key2.as<uint64_t>(), pay2.as<uint32_t>(), m, bb + bf, s));
+            LIFE_TRY(radix_sort_pairs(key2, pay2, m, 0, bb + bf, s));
             head_flag_kernel<<<grid1d(m), 256, 0, s>>>(key2.as<uint64_t>(), m, head.as<int32_t>());
             LIFE_CHECK_LAUNCH();
             LIFE_TRY(exclusive_scan_i32(head.as<int32_t>(), uidx.as<int32_t>(), m, s));
@@ -856,7 +857,7 @@ life_status build_tile_layout(life_index_s* ix, cudaStream_t s) {
         if (m > 0) {
             wc_key_kernel<<<grid1d(m), 256, 0, s>>>(skey.as<uint64_t>(), m, bf, key2.as<uint64_t>(), pay2.as<uint32_t>());
             LIFE_CHECK_LAUNCH();
-            LIFE_TRY(radix_sort_pairs(key2.as<uint64_t>(), pay2.as<uint32_t>(), m, nbits64(H.n_tiles) + 16 + bf, s));
+            LIFE_TRY(radix_sort_pairs(key2, pay2, m, bf, nbits64(H.n_tiles) + 16 + bf, s));
             if (L.vbytes == 4)
                 wc_stream_kernel<<<grid1d(m), 256, 0, s>>>(key2.as<uint64_t>(), pay2.as<uint32_t>(), m, bf,
                                                            L.fl.as<uint16_t>(), L.val.as<float>(), L.n_sub, n_wsegs, 1,
