@@ -349,7 +349,7 @@ template <class VT>
 __global__ void __launch_bounds__(MG_THREADS)
 merge_layout_kernel(const uint64_t* __restrict__ key, const uint32_t* __restrict__ payload, int64_t n,
                     const int32_t* __restrict__ offset, int32_t m, int sa, int sv, uint64_t amask, uint64_t fmask,
-                    int32_t nv, uint64_t* __restrict__ ukey, float* __restrict__ uval, uint16_t* __restrict__ atom16,
+                    int32_t nv, float* __restrict__ uval, uint16_t* __restrict__ atom16,
                     int32_t* __restrict__ fasc, VT* __restrict__ valout, int32_t* __restrict__ vox_ptr) {
     __shared__ int32_t wsum[MG_ROUNDS][MG_THREADS / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -392,12 +392,14 @@ merge_layout_kernel(const uint64_t* __restrict__ key, const uint32_t* __restrict
         for (int64_t q = i + 1; q < n && key[q] == k[j]; ++q) sum += (double)__uint_as_float(payload[q]);
         const float x = (float)sum;
         const int32_t v = (int32_t)(k[j] >> sv);
-        ukey[pos] = k[j];
-        uval[pos] = x;
         atom16[pos] = (uint16_t)((k[j] >> sa) & amask);
         fasc[pos] = (int32_t)(k[j] & fmask);
-        if constexpr (sizeof(VT) == 2) valout[pos] = __float2bfloat16_rn(x);
-        else valout[pos] = x;
+        if constexpr (sizeof(VT) == 2) {
+            valout[pos] = __float2bfloat16_rn(x);
+            uval[pos] = x;
+        } else {
+            valout[pos] = x;
+        }
         const int32_t vp = i == 0 ? -1 : (int32_t)(kp[j] >> sv);
         for (int32_t q = vp + 1; q <= v; ++q) vox_ptr[q] = pos;
         if (pos == m - 1)
@@ -470,10 +472,9 @@ life_status build_voxel_layout(life_index_s* ix, const int32_t* atom, const int3
         LIFE_CUDA_TRY(cudaStreamSynchronize(s));
     }
     ix->nnz = m;
-    LIFE_TRY(ix->ukey.alloc(sizeof(uint64_t) * (size_t)m));
-    LIFE_TRY(ix->uval.alloc(sizeof(float) * (size_t)m));
     VoxelLayout& L = ix->vox;
     const bool bf16 = ix->precision == LIFE_BF16;
+    if (bf16) LIFE_TRY(ix->uval.alloc(sizeof(float) * (size_t)m));
     LIFE_TRY(L.vox_ptr.alloc(sizeof(int32_t) * ((size_t)ix->nv + 1)));
     LIFE_TRY(L.atom.alloc(sizeof(uint16_t) * (size_t)m));
     LIFE_TRY(L.fasc.alloc(sizeof(int32_t) * (size_t)m));
@@ -483,12 +484,12 @@ life_status build_voxel_layout(life_index_s* ix, const int32_t* atom, const int3
     } else if (bf16) {
         merge_layout_kernel<<<(unsigned)nblk, MG_THREADS, 0, s>>>(
             keys.as<uint64_t>(), pay.as<uint32_t>(), n, offset.as<int32_t>(), m, sa, sv, (1ull << ba) - 1,
-            (1ull << bf) - 1, ix->nv, ix->ukey.as<uint64_t>(), ix->uval.as<float>(), L.atom.as<uint16_t>(),
+            (1ull << bf) - 1, ix->nv, ix->uval.as<float>(), L.atom.as<uint16_t>(),
             L.fasc.as<int32_t>(), L.val.as<__nv_bfloat16>(), L.vox_ptr.as<int32_t>());
     } else {
         merge_layout_kernel<<<(unsigned)nblk, MG_THREADS, 0, s>>>(
             keys.as<uint64_t>(), pay.as<uint32_t>(), n, offset.as<int32_t>(), m, sa, sv, (1ull << ba) - 1,
-            (1ull << bf) - 1, ix->nv, ix->ukey.as<uint64_t>(), ix->uval.as<float>(), L.atom.as<uint16_t>(),
+            (1ull << bf) - 1, ix->nv, nullptr, L.atom.as<uint16_t>(),
             L.fasc.as<int32_t>(), L.val.as<float>(), L.vox_ptr.as<int32_t>());
     }
     LIFE_CHECK_LAUNCH();
@@ -498,47 +499,49 @@ life_status build_voxel_layout(life_index_s* ix, const int32_t* atom, const int3
 
 // ------------------------------------------------------------ re-sorting
 
+// Voxel of each entry of the merged list (one warp per voxel).
+__global__ void entry_voxel_kernel(const int32_t* __restrict__ vox_ptr, int32_t nv, int32_t* __restrict__ voxel) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t v = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; v < nv; v += warps)
+        for (int32_t i = vox_ptr[v] + lane; i < vox_ptr[v + 1]; i += 32) voxel[i] = (int32_t)v;
+}
+
 // Re-keys the merged (v, a, f) list in another order; payload = merged position.
-__global__ void rekey_kernel(const uint64_t* __restrict__ ukey, int64_t m, int order, int bv, int ba, int bf,
+__global__ void rekey_kernel(const int32_t* __restrict__ voxel, const uint16_t* __restrict__ atom,
+                             const int32_t* __restrict__ fasc, int64_t m, int order, int bv, int ba, int bf,
                              uint64_t* __restrict__ key, uint32_t* __restrict__ payload) {
-    const int sa = bf, sv = bf + ba;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t k = ukey[i];
-        const uint64_t v = k >> sv, a = (k >> sa) & ((1ull << ba) - 1), f = k & ((1ull << bf) - 1);
-        uint64_t nk;
-        if (order == LIFE_LAYOUT_FIBER) nk = (f << (bv + ba)) | (v << ba) | a;
-        else if (order == LIFE_LAYOUT_ATOM) nk = (a << (bv + bf)) | (v << bf) | f;
-        else nk = k;
-        key[i] = nk;
+        const uint64_t v = (uint64_t)voxel[i], a = atom[i], f = (uint64_t)fasc[i];
+        key[i] = order == LIFE_LAYOUT_FIBER ? (f << (bv + ba)) | (v << ba) | a : (a << (bv + bf)) | (v << bf) | f;
         payload[i] = (uint32_t)i;
     }
 }
 
-__global__ void gather_export_kernel(const uint64_t* __restrict__ ukey, const float* __restrict__ uval,
-                                     const uint32_t* __restrict__ perm, int64_t m, int ba, int bf,
-                                     int32_t* __restrict__ atom, int32_t* __restrict__ voxel,
-                                     int32_t* __restrict__ fasc, float* __restrict__ val) {
-    const int sa = bf, sv = bf + ba;
+__global__ void gather_export_kernel(const int32_t* __restrict__ vsrc, const uint16_t* __restrict__ asrc,
+                                     const int32_t* __restrict__ fsrc, const float* __restrict__ xsrc,
+                                     const uint32_t* __restrict__ perm, int64_t m, int32_t* __restrict__ atom,
+                                     int32_t* __restrict__ voxel, int32_t* __restrict__ fasc,
+                                     float* __restrict__ val) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t p = perm ? perm[i] : (uint32_t)i;
-        const uint64_t k = ukey[p];
-        if (atom) atom[i] = (int32_t)((k >> sa) & ((1ull << ba) - 1));
-        if (voxel) voxel[i] = (int32_t)(k >> sv);
-        if (fasc) fasc[i] = (int32_t)(k & ((1ull << bf) - 1));
-        if (val) val[i] = uval[p];
+        if (atom) atom[i] = asrc[p];
+        if (voxel) voxel[i] = vsrc[p];
+        if (fasc) fasc[i] = fsrc[p];
+        if (val) val[i] = xsrc[p];
     }
 }
 
 // Sorted permutation of the merged list for a layout (NULL perm = voxel order).
-static life_status layout_perm(life_index_s* ix, int layout, TmpBuf& perm, cudaStream_t s) {
+static life_status layout_perm(life_index_s* ix, int layout, const int32_t* voxel, TmpBuf& perm, cudaStream_t s) {
     const int64_t m = ix->nnz;
     if (layout == LIFE_LAYOUT_VOXEL || m == 0) return LIFE_OK;
     TmpBuf keys;
     LIFE_TRY(keys.alloc(sizeof(uint64_t) * m, s));
     LIFE_TRY(perm.alloc(sizeof(uint32_t) * m, s));
     const int bv = ix->key_bits_v, ba = ix->key_bits_a, bf = ix->key_bits_f;
-    rekey_kernel<<<grid_for(m), 256, 0, s>>>(ix->ukey.as<uint64_t>(), m, layout, bv, ba, bf, keys.as<uint64_t>(),
-                                             perm.as<uint32_t>());
+    rekey_kernel<<<grid_for(m), 256, 0, s>>>(voxel, ix->vox.atom.as<uint16_t>(), ix->vox.fasc.as<int32_t>(), m, layout,
+                                             bv, ba, bf, keys.as<uint64_t>(), perm.as<uint32_t>());
     LIFE_CHECK_LAUNCH();
     // the list is in (v, a, f) order and the sort stable: only the leading field of the
     // new order, the atom or the fascicle, has to be sorted
@@ -555,10 +558,15 @@ life_status export_layout(life_index_s* ix, int layout, int32_t* atom, int32_t* 
     }
     const int64_t m = ix->nnz;
     if (m == 0) return LIFE_OK;
-    TmpBuf perm;
-    LIFE_TRY(layout_perm(ix, layout, perm, s));
-    gather_export_kernel<<<grid_for(m), 256, 0, s>>>(ix->ukey.as<uint64_t>(), ix->uval.as<float>(),
-                                                     perm.as<uint32_t>(), m, ix->key_bits_a, ix->key_bits_f, atom,
+    TmpBuf vox, perm;
+    LIFE_TRY(vox.alloc(sizeof(int32_t) * m, s));
+    entry_voxel_kernel<<<grid_for((int64_t)ix->nv * 32), 256, 0, s>>>(ix->vox.vox_ptr.as<int32_t>(), ix->nv,
+                                                                      vox.as<int32_t>());
+    LIFE_CHECK_LAUNCH();
+    LIFE_TRY(layout_perm(ix, layout, vox.as<int32_t>(), perm, s));
+    const float* x = ix->precision == LIFE_BF16 ? ix->uval.as<float>() : ix->vox.val.as<float>();
+    gather_export_kernel<<<grid_for(m), 256, 0, s>>>(vox.as<int32_t>(), ix->vox.atom.as<uint16_t>(),
+                                                     ix->vox.fasc.as<int32_t>(), x, perm.as<uint32_t>(), m, atom,
                                                      voxel, fasc, val);
     LIFE_CHECK_LAUNCH();
     LIFE_CUDA_TRY(cudaStreamSynchronize(s));

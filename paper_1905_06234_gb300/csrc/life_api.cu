@@ -231,12 +231,12 @@ extern "C" life_status life_index_get_info(life_index idx, life_index_info* out)
     I.sparse_dsc = idx->tile.sparse ? 1 : 0;
     I.n_tiles = idx->tile.n_tiles;
     I.n_bricks = idx->tile.n_bricks;
-    const DevBuf* bufs[] = {&idx->ukey, &idx->uval, &idx->voxel_ijk, &idx->vox.vox_ptr, &idx->vox.atom,
+    const DevBuf* bufs[] = {&idx->uval, &idx->voxel_ijk, &idx->vox.vox_ptr, &idx->vox.atom,
                             &idx->vox.fasc, &idx->vox.val, &idx->atoml.voxel, &idx->atoml.fasc, &idx->atoml.val,
                             &idx->atoml.chunk_beg, &idx->atoml.chunk_atom, &idx->atoml.atom_chunk,
                             &idx->tile.tile_vox, &idx->tile.chunk_ptr, &idx->tile.brick_tile_ptr,
                             &idx->tile.brick_fasc_ptr, &idx->tile.brick_fasc, &idx->tile.brick_order,
-                            &idx->tile.va, &idx->tile.soff, &idx->tile.fl, &idx->tile.val, &idx->tile.wkey,
+                            &idx->tile.soff, &idx->tile.fl, &idx->tile.val, &idx->tile.wkey,
                             &idx->tile.wfl, &idx->tile.wval, &idx->tile.wseg_ptr, &idx->tile.wb_src,
                             &idx->tile.wb_ptr, &idx->tile.wb, &idx->tile.brick_cv, &idx->tile.tile_amax, &idx->red,
                             &idx->tile.c_soff, &idx->tile.c_fl, &idx->tile.c_val, &idx->tile.c_chunk_end,

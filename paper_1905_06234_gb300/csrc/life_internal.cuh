@@ -71,6 +71,10 @@ struct DevBuf {
         bytes = n;
         return LIFE_OK;
     }
+    void swap(DevBuf& o) {
+        std::swap(p, o.p);
+        std::swap(bytes, o.bytes);
+    }
     template <class T> T* as() const { return static_cast<T*>(p); }
 };
 
@@ -149,7 +153,6 @@ struct TileLayout {
     DevBuf brick_fasc_ptr;   // int32 [n_bricks + 1] offsets into brick_fasc
     DevBuf brick_fasc;       // int32 [sum] global fascicle id of each brick-local fascicle
     DevBuf brick_order;      // int32 [n_bricks] bricks by decreasing entry count
-    DevBuf va;               // uint16 [n_nnz]: row | (atom << 7)
     DevBuf soff;             // uint16 [n_nnz]: byte offset of (row, atom mod 128) in a DSC S chunk | 0x8000
                              // if the entry has the same (atom, row) as the previous one
     // WC streams, ordered (tile, row quarter, atom, row, fascicle)
@@ -233,8 +236,7 @@ struct life_index_s {
     int32_t key_bits_v = 0, key_bits_a = 0, key_bits_f = 0;
     int device = 0;
     int num_sms = 0;
-    life::DevBuf ukey;          // uint64 [nnz] merged keys in (v, a, f) order
-    life::DevBuf uval;          // float [nnz] merged values
+    life::DevBuf uval;          // float [nnz] merged values of a BF16 index (an FP32 one's are vox.val)
     life::DevBuf voxel_ijk;     // int32 [Nv*3] copy (optional)
     life::VoxelLayout vox;
     life::AtomLayout atoml;

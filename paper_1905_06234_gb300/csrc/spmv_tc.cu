@@ -14,108 +14,22 @@
 // are K-major, no-swizzle core-matrix layouts in shared memory.
 #include <algorithm>
 #include <cstring>
-#include <numeric>
 #include <type_traits>
 #include <vector>
 
-#include "life_internal.cuh"
+#include "tile_layout.cuh"
 #include "tc_ptx.cuh"
 
 namespace life {
 
 using namespace ptx;
 
-constexpr int SUB = 32;                  // atoms per WC segment (offset granularity of the WC streams)
-constexpr int DKC = 128;                 // atoms per DSC K chunk (offset granularity of the DSC stream)
-constexpr int ZW = 33;                   // row stride (floats) of a WC scatter warp's 32 x 32 Z tile
-constexpr uint16_t CONT = 0x8000;        // entry continues the previous entry's (atom, row)
 constexpr uint64_t WAIT_LIMIT = 2000000000ull; // ns before a wait gives up
-
-static int nbits64(int64_t n) {
-    if (n <= 1) return 0;
-    uint64_t x = (uint64_t)(n - 1);
-    int b = 0;
-    while (x) { ++b; x >>= 1; }
-    return b;
-}
 
 static unsigned grid1d(int64_t n, int threads = 256) {
     int64_t b = (n + threads - 1) / threads;
     int64_t cap = (int64_t)device_sm_count() * 32;
     return (unsigned)std::max<int64_t>(1, std::min(b, cap));
-}
-
-// ============================================================ layout build
-
-// The (atom, row) cell part (16 bits) of the DSC sort key: the 128-atom chunk,
-// then the cell's place in the chunk's S operand (8-row group, 8-atom group, row
-// mod 8, atom mod 8), i.e. the order of its byte offset there.  An 8 x 8 group of
-// cells spans the 32 shared-memory banks once, so the run sums that the lanes of a
-// warp store at the same time fall on more distinct banks than in (atom, row)
-// order.  Runs (entries of one cell) stay contiguous; Na < 512.
-__host__ __device__ inline uint64_t cell_key(uint64_t a, uint64_t row) {
-    return ((a >> 7) << 14) | ((row >> 3) << 10) | (((a >> 3) & 15u) << 6) | ((row & 7u) << 3) | (a & 7u);
-}
-__host__ __device__ inline void cell_of_key(uint64_t ck, uint32_t& a, uint32_t& row) {
-    a = (uint32_t)((((ck >> 14) & 3u) << 7) | (((ck >> 6) & 15u) << 3) | (ck & 7u));
-    row = (uint32_t)((((ck >> 10) & 15u) << 3) | ((ck >> 3) & 7u));
-}
-
-// key = tile | cell_key(atom, row) | fascicle  (payload: position in the merged list)
-__global__ void tile_key_kernel(const uint64_t* __restrict__ ukey, int64_t m, int sa, int sv, uint64_t amask,
-                                uint64_t fmask, int bf, const int32_t* __restrict__ vox_tile,
-                                const int32_t* __restrict__ vox_row, uint64_t* __restrict__ key,
-                                uint32_t* __restrict__ pay) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t k = ukey[i];
-        const uint64_t v = k >> sv, a = (k >> sa) & amask, f = k & fmask;
-        const uint64_t t = (uint64_t)vox_tile[v], row = (uint64_t)vox_row[v];
-        key[i] = (t << (16 + bf)) | (cell_key(a, row) << bf) | f;
-        pay[i] = (uint32_t)i;
-    }
-}
-
-// key2 = brick | fascicle (payload: position in tile order)
-__global__ void brick_key_kernel(const uint64_t* __restrict__ skey, int64_t m, int bf,
-                                 const int32_t* __restrict__ tile_brick, uint64_t* __restrict__ key2,
-                                 uint32_t* __restrict__ pay2) {
-    const uint64_t fmask = (1ull << bf) - 1;
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t k = skey[j];
-        const uint64_t t = k >> (16 + bf);
-        key2[j] = ((uint64_t)tile_brick[t] << bf) | (k & fmask);
-        pay2[j] = (uint32_t)j;
-    }
-}
-
-__global__ void head_flag_kernel(const uint64_t* __restrict__ key, int64_t m, int32_t* __restrict__ head) {
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x)
-        head[j] = (j == 0 || key[j] != key[j - 1]) ? 1 : 0;
-}
-
-// Distinct fascicles per brick: the brick's table and its offsets (gap-filled).
-__global__ void brick_fasc_kernel(const uint64_t* __restrict__ key2, int64_t m, int bf,
-                                  const int32_t* __restrict__ head, const int32_t* __restrict__ uidx, int32_t nb,
-                                  int32_t n_unique, int32_t* __restrict__ bptr, int32_t* __restrict__ bfasc) {
-    const uint64_t fmask = (1ull << bf) - 1;
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t k = key2[j];
-        const int32_t b = (int32_t)(k >> bf);
-        if (head[j]) bfasc[uidx[j]] = (int32_t)(k & fmask);
-        const int32_t bp = j == 0 ? -1 : (int32_t)(key2[j - 1] >> bf);
-        for (int32_t q = bp + 1; q <= b; ++q) bptr[q] = uidx[j];
-        if (j == m - 1)
-            for (int32_t q = b + 1; q <= nb; ++q) bptr[q] = n_unique;
-    }
-}
-
-// wb_src[wb_ptr[b] + i] = brick_fasc[brick_fasc_ptr[b] + i], padding slots -1 (one block per brick).
-__global__ void wb_src_kernel(const int32_t* __restrict__ bptr, const int32_t* __restrict__ bfasc,
-                              const int32_t* __restrict__ wptr, int32_t nb, int32_t* __restrict__ wsrc) {
-    for (int32_t b = blockIdx.x; b < nb; b += gridDim.x) {
-        const int32_t f0 = bptr[b], n = bptr[b + 1] - f0, o = wptr[b], np = wptr[b + 1] - o;
-        for (int32_t i = threadIdx.x; i < np; i += blockDim.x) wsrc[o + i] = i < n ? bfasc[f0 + i] : -1;
-    }
 }
 
 __device__ __forceinline__ float gather_slot(const float* __restrict__ w, int32_t id) {
@@ -170,21 +84,6 @@ __global__ void __launch_bounds__(256) x_amax_kernel(const float* __restrict__ x
 // the same S values up to the association of a run's FP32 sum.
 
 enum : uint32_t { DSC_MODE_NONE = 0, DSC_MODE_FULL = 1, DSC_MODE_COMPACT = 2 };
-
-struct SparseCtl {
-    unsigned long long n_live;        // real slots with x != 0 seen by this call's gather
-    unsigned long long n_live_cmp;    // that count when the compacted stream was built
-    unsigned long long n_compactions; // compacted-stream rebuilds so far
-    unsigned long long n_compact_calls;  // DSC calls that streamed the compacted entries
-    unsigned long long n_calls;       // DSC calls that went through the decision
-    uint32_t stale;                   // some slot with x != 0 lies outside L
-    uint32_t mode;                    // DSC_MODE_* of the current call
-    uint32_t compact_now;             // the current call rebuilds the compacted stream
-    uint32_t have;                    // a compacted stream exists
-    uint32_t gather_done;             // blocks of the gather finished (the last one decides)
-    uint32_t since;                   // decisions since the last rebuild
-    uint32_t gap;                     // decisions a rebuild for a stale live set must wait (backoff)
-};
 
 // Thresholds of the decision: the compacted stream is used only while the live
 // slots are at most DENSE_FRAC of all slots, and rebuilt once the live count has
@@ -392,552 +291,6 @@ __global__ void __launch_bounds__(CMP_THREADS) cmp_rebuild_kernel(CompactArgs C)
     }
 }
 
-// cv[b] = (largest number of WC entries of one brick-local fascicle of brick b) x
-// (largest |val| of the brick), rounded up: it bounds Σ|val| over the entries of
-// any fascicle of the brick.  Integer counts and maxima, so the result does not
-// depend on the order of the atomics.  Dynamic shared memory: max_fb counters.
-__global__ void brick_cv_kernel(const int32_t* __restrict__ btile, const int32_t* __restrict__ bfptr,
-                                const int32_t* __restrict__ wseg_ptr, int32_t seg_per_tile,
-                                const uint16_t* __restrict__ wfl, const __nv_bfloat16* __restrict__ wval,
-                                int32_t nb, float* __restrict__ cv) {
-    extern __shared__ int32_t cnt[];
-    __shared__ uint32_t vmax_bits, cmax;
-    for (int32_t b = blockIdx.x; b < nb; b += gridDim.x) {
-        const int32_t nfb = bfptr[b + 1] - bfptr[b];
-        for (int32_t i = threadIdx.x; i < nfb; i += blockDim.x) cnt[i] = 0;
-        if (threadIdx.x == 0) vmax_bits = cmax = 0u;
-        __syncthreads();
-        const int32_t j0 = wseg_ptr[(int64_t)btile[b] * seg_per_tile], j1 = wseg_ptr[(int64_t)btile[b + 1] * seg_per_tile];
-        uint32_t vm = 0u;
-        for (int32_t j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
-            atomicAdd(&cnt[wfl[j] >> 2], 1);
-            vm = max(vm, __float_as_uint(__bfloat162float(wval[j])) & 0x7FFFFFFFu);
-        }
-        for (int o = 16; o > 0; o >>= 1) vm = max(vm, __shfl_xor_sync(0xffffffffu, vm, o));
-        if ((threadIdx.x & 31) == 0) atomicMax(&vmax_bits, vm);
-        __syncthreads();
-        uint32_t cm = 0u;
-        for (int32_t i = threadIdx.x; i < nfb; i += blockDim.x) cm = max(cm, (uint32_t)cnt[i]);
-        for (int o = 16; o > 0; o >>= 1) cm = max(cm, __shfl_xor_sync(0xffffffffu, cm, o));
-        if ((threadIdx.x & 31) == 0) atomicMax(&cmax, cm);
-        __syncthreads();
-        if (threadIdx.x == 0) cv[b] = __fmul_ru((float)cmax, __uint_as_float(vmax_bits));
-        __syncthreads();
-    }
-}
-
-// Brick-local fascicle number of each entry, scattered back to tile order.
-// uidx is the exclusive scan of the head flags, so an entry that repeats its
-// predecessor's (brick, fascicle) belongs to unique index uidx - 1.
-__global__ void local_fasc_kernel(const uint64_t* __restrict__ key2, const uint32_t* __restrict__ pay2, int64_t m,
-                                  int bf, const int32_t* __restrict__ head, const int32_t* __restrict__ uidx,
-                                  const int32_t* __restrict__ bptr, uint16_t* __restrict__ fl) {
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t b = (int32_t)(key2[j] >> bf);
-        const int32_t u = uidx[j] + head[j] - 1;
-        fl[pay2[j]] = (uint16_t)(4 * (u - bptr[b]));  // byte offset in the brick's weight table
-    }
-}
-
-// Stored values: BF16 (rounded once from the merged FP32 value) or FP32 (as merged).
-__device__ __forceinline__ void store_val(__nv_bfloat16* p, float x) { *p = __float2bfloat16_rn(x); }
-__device__ __forceinline__ void store_val(float* p, float x) { *p = x; }
-__device__ __forceinline__ float load_val(const __nv_bfloat16* p) { return __bfloat162float(*p); }
-__device__ __forceinline__ float load_val(const float* p) { return *p; }
-
-// Entry streams in tile order, the continuation flag, and the chunk offsets.
-template <class VT>
-__global__ void tile_stream_kernel(const uint64_t* __restrict__ skey, const uint32_t* __restrict__ spay, int64_t m,
-                                   int bf, const float* __restrict__ uval, int32_t n_c, int64_t n_segs,
-                                   uint16_t* __restrict__ va, uint16_t* __restrict__ soff,
-                                   uint16_t* __restrict__ fl, VT* __restrict__ val,
-                                   int32_t* __restrict__ chunk_ptr) {
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t k = skey[j];
-        const uint64_t t = k >> (16 + bf);
-        uint32_t a, row;
-        cell_of_key((k >> bf) & 0xFFFFu, a, row);
-        va[j] = (uint16_t)(row | (a << 7));
-        // byte offset of (row, atom) in an S chunk (< 32768), with the continuation bit
-        const bool cont = j > 0 && (skey[j - 1] >> bf) == (k >> bf);
-        soff[j] = (uint16_t)(ptx::kmajor_off(row, a & 127u, (128 / 8) * 128) | (cont ? CONT : 0u));
-        store_val(val + j, uval[spay[j]]);
-        // the chunk is the top of the cell key
-        const int64_t seg = (int64_t)t * n_c + (a >> 7);
-        int64_t segp = -1;
-        if (j > 0) {
-            const uint64_t kp = skey[j - 1];
-            segp = (int64_t)(kp >> (16 + bf)) * n_c + (int64_t)((kp >> (14 + bf)) & 3u);
-        }
-        for (int64_t q = segp + 1; q <= seg; ++q) chunk_ptr[q] = (int32_t)j;
-        if (j == m - 1)
-            for (int64_t q = seg + 1; q <= n_segs; ++q) chunk_ptr[q] = (int32_t)m;
-    }
-}
-
-// WC order: key3 = tile | row quarter | atom | row mod 32 | fascicle (payload:
-// position in the DSC stream)
-__global__ void wc_key_kernel(const uint64_t* __restrict__ skey, int64_t m, int bf, uint64_t* __restrict__ key3,
-                              uint32_t* __restrict__ pay3) {
-    const uint64_t fmask = (1ull << bf) - 1;
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t k = skey[j];
-        uint32_t a32, r32;
-        cell_of_key((k >> bf) & 0xFFFFu, a32, r32);
-        const uint64_t t = k >> (16 + bf), a = a32, row = r32;
-        key3[j] = (t << (16 + bf)) | ((row >> 5) << (14 + bf)) | (a << (5 + bf)) | ((row & 31u) << bf) | (k & fmask);
-        pay3[j] = (uint32_t)j;
-    }
-}
-
-template <class VT>
-__global__ void wc_stream_kernel(const uint64_t* __restrict__ key3, const uint32_t* __restrict__ pay3, int64_t m,
-                                 int bf, const uint16_t* __restrict__ fl, const VT* __restrict__ val,
-                                 int32_t n_sub, int64_t n_segs, int atom_major, uint16_t* __restrict__ wkey,
-                                 uint16_t* __restrict__ wfl, VT* __restrict__ wval, int32_t* __restrict__ wseg_ptr) {
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t k = key3[j];
-        const uint32_t src = pay3[j];
-        const uint64_t t = k >> (16 + bf), q = (k >> (14 + bf)) & 3u, a = (k >> (5 + bf)) & 511u,
-                       r32 = (k >> bf) & 31u;
-        // byte offsets: of the entry's (row, atom) cell in a scatter warp's Z tile
-        // (row-major, or atom-major for the FP32-storage kernel) and of its
-        // fascicle in the brick table (< 15872 fascicles: fits 16 bits)
-        const uint32_t cell = atom_major ? (uint32_t)(a & 31u) * ZW + (uint32_t)r32 : (uint32_t)r32 * ZW + (uint32_t)(a & 31u);
-        wkey[j] = (uint16_t)(4u * cell);
-        wfl[j] = fl[src];
-        wval[j] = val[src];
-        const int64_t seg = ((int64_t)t * 4 + (int64_t)q) * n_sub + (int64_t)(a >> 5);
-        int64_t segp = -1;
-        if (j > 0) {
-            const uint64_t kp = key3[j - 1];
-            segp = ((int64_t)(kp >> (16 + bf)) * 4 + (int64_t)((kp >> (14 + bf)) & 3u)) * n_sub +
-                   (int64_t)(((kp >> (5 + bf)) & 511u) >> 5);
-        }
-        for (int64_t q2 = segp + 1; q2 <= seg; ++q2) wseg_ptr[q2] = (int32_t)j;
-        if (j == m - 1)
-            for (int64_t q2 = seg + 1; q2 <= n_segs; ++q2) wseg_ptr[q2] = (int32_t)m;
-    }
-}
-
-__global__ void fill_kernel(int32_t* p, int64_t n, int32_t v) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) p[i] = v;
-}
-
-// Bits of the largest Σ|val| over the entries of one (atom, voxel) run of the DSC
-// stream (a run starts at an entry without the continuation flag): with max |x|
-// it bounds every S value of a DSC.
-template <class VT>
-__global__ void run_vmax_kernel(const uint16_t* __restrict__ soff, const VT* __restrict__ val, int64_t m,
-                                uint32_t* __restrict__ out) {
-    uint32_t best = 0u;
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
-        if (soff[j] & CONT) continue;
-        float sum = fabsf(load_val(val + j));
-        for (int64_t k = j + 1; k < m && (soff[k] & CONT); ++k) sum += fabsf(load_val(val + k));
-        best = max(best, __float_as_uint(sum));
-    }
-    for (int o = 16; o > 0; o >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, o));
-    if ((threadIdx.x & 31) == 0 && best) atomicMax(out, best);
-}
-
-// Tensor-memory columns the FP32-storage WC needs: D's FP16 hi and lo parts for
-// each 128-atom block (np/2 columns each) and three 64-column Z slots.
-__host__ __device__ inline int wc32_tmem_cols(int np, int kp) { return (kp / 128) * np + 3 * 64; }
-
-struct HostTiles {
-    std::vector<int32_t> tile_vox, vox_tile, vox_row, tile_brick, brick_tile_ptr;
-    int64_t n_tiles = 0, n_bricks = 0;
-};
-
-// Groups voxels into bricks (spatial bx x by x bz boxes when coordinates are
-// known, else runs of bx*by*bz consecutive voxel ids) and each brick into
-// 128-voxel tiles.  shape[g] is the brick shape of group g (one group, or one per
-// problem of a batch).  For the combined index of a batch, bricks never mix
-// problems: the problem is the leading part of the brick key, and voxel-id runs
-// restart at each problem.
-struct BrickShape {
-    int x, y, z;
-    int64_t volume() const { return (int64_t)x * y * z; }
-};
-
-static void assign_tiles(int32_t nv, const std::vector<int32_t>& ijk, const std::vector<BrickShape>& shape,
-                         const BatchInfo& bi, HostTiles& H) {
-    std::vector<int64_t> bkey(nv);
-    const bool grouped = !bi.vox_group.empty();
-    int32_t mx[3] = {0, 0, 0};
-    if (!ijk.empty())
-        for (int32_t v = 0; v < nv; ++v)
-            for (int d = 0; d < 3; ++d) mx[d] = std::max(mx[d], ijk[3 * v + d]);
-    for (int32_t v = 0; v < nv; ++v) {
-        const int g = grouped ? bi.vox_group[v] : 0;
-        const BrickShape& sh = shape[g];
-        if (!ijk.empty()) {
-            const int64_t nbx = mx[0] / sh.x + 1, nby = mx[1] / sh.y + 1;
-            bkey[v] = ((int64_t)(ijk[3 * v + 2] / sh.z) * nby + ijk[3 * v + 1] / sh.y) * nbx + ijk[3 * v] / sh.x;
-        } else {
-            bkey[v] = (grouped ? v - bi.vox_off[g] : v) / sh.volume();
-        }
-        if (grouped) bkey[v] |= (int64_t)g << 40;
-    }
-    std::vector<int32_t> order(nv);
-    std::iota(order.begin(), order.end(), 0);
-    std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return bkey[x] < bkey[y]; });
-    H.vox_tile.assign(nv, 0);
-    H.vox_row.assign(nv, 0);
-    H.tile_vox.clear();
-    H.tile_brick.clear();
-    H.brick_tile_ptr.assign(1, 0);
-    int64_t i = 0;
-    int32_t brick = 0;
-    while (i < nv) {
-        int64_t j = i;
-        while (j < nv && bkey[order[j]] == bkey[order[i]]) ++j;
-        for (int64_t s = i; s < j; s += TILE_V) {
-            const int32_t t = (int32_t)(H.tile_vox.size() / TILE_V);
-            for (int r = 0; r < TILE_V; ++r) {
-                const int64_t q = s + r;
-                if (q < j) {
-                    const int32_t v = order[q];
-                    H.tile_vox.push_back(v);
-                    H.vox_tile[v] = t;
-                    H.vox_row[v] = r;
-                } else {
-                    H.tile_vox.push_back(-1);
-                }
-            }
-            H.tile_brick.push_back(brick);
-        }
-        H.brick_tile_ptr.push_back((int32_t)(H.tile_vox.size() / TILE_V));
-        ++brick;
-        i = j;
-    }
-    H.n_tiles = (int64_t)H.tile_vox.size() / TILE_V;
-    H.n_bricks = brick;
-}
-
-template <class T>
-static life_status upload(DevBuf& dst, const std::vector<T>& src, cudaStream_t s) {
-    LIFE_TRY(dst.alloc(sizeof(T) * std::max<size_t>(src.size(), 1)));
-    if (!src.empty())
-        LIFE_CUDA_TRY(cudaMemcpyAsync(dst.p, src.data(), sizeof(T) * src.size(), cudaMemcpyHostToDevice, s));
-    return LIFE_OK;
-}
-
-life_status build_tile_layout(life_index_s* ix, cudaStream_t s) {
-    TileLayout& L = ix->tile;
-    if (ix->na > 512 || ix->nt > 128) {
-        set_error("tensor-core path supports Na <= 512 and Ntheta <= 128 (got %d, %d)", ix->na, ix->nt);
-        return LIFE_ENOTSUP;
-    }
-    if (ix->key_bits_f > 32) {
-        set_error("tensor-core path: too many fascicles");
-        return LIFE_ENOTSUP;
-    }
-    if (ix->precision == LIFE_FP32 && ix->na > 384) {
-        // D's two FP16 parts (Na/2 columns each) and the 128-column accumulator share
-        // the 512 tensor-memory columns of an SM
-        set_error("FP32 tensor-core DSC supports Na <= 384 (got %d)", ix->na);
-        return LIFE_ENOTSUP;
-    }
-    if (ix->precision == LIFE_FP32 && ix->sparse_dsc) {
-        set_error("the live-entry DSC stream is built for BF16 storage only");
-        return LIFE_ENOTSUP;
-    }
-    const int64_t m = ix->nnz;
-    L.vbytes = ix->precision == LIFE_FP32 ? 4 : 2;
-    L.np = (ix->nt + 15) / 16 * 16;
-    L.kp = (ix->na + 127) / 128 * 128;   // whole 128-atom DSC chunks
-    // the FP32-storage WC holds D's FP16 parts (np columns per 128-atom block) and a
-    // ring of three 64-column Z slots in tensor memory; beyond that WC runs on the
-    // CUDA cores
-    L.wc_stream = L.vbytes == 2 || wc32_tmem_cols(L.np, L.kp) <= 512;
-    L.n_sub = L.kp / SUB;
-    const int bf = ix->key_bits_f, ba = ix->key_bits_a, sa = bf, sv = bf + ba;
-    std::vector<int32_t> ijk;
-    if (ix->voxel_ijk.p) {
-        ijk.resize((size_t)ix->nv * 3);
-        LIFE_CUDA_TRY(cudaMemcpyAsync(ijk.data(), ix->voxel_ijk.p, sizeof(int32_t) * ijk.size(), cudaMemcpyDeviceToHost, s));
-        LIFE_CUDA_TRY(cudaStreamSynchronize(s));
-    }
-    TmpBuf skey, spay;
-    LIFE_TRY(skey.alloc(sizeof(uint64_t) * std::max<int64_t>(m, 1), s));
-    LIFE_TRY(spay.alloc(sizeof(uint32_t) * std::max<int64_t>(m, 1), s));
-    HostTiles H;
-    std::vector<int32_t> hbptr;
-    DevBuf d_vox_tile, d_vox_row, d_tile_brick;
-    TmpBuf key2, pay2, head, uidx;
-    LIFE_TRY(key2.alloc(sizeof(uint64_t) * std::max<int64_t>(m, 1), s));
-    LIFE_TRY(pay2.alloc(sizeof(uint32_t) * std::max<int64_t>(m, 1), s));
-    LIFE_TRY(head.alloc(sizeof(int32_t) * std::max<int64_t>(m, 1), s));
-    LIFE_TRY(uidx.alloc(sizeof(int32_t) * std::max<int64_t>(m, 1), s));
-    int32_t n_unique = 0;
-    bool ok = false;
-    // Every group starts from B0^3 bricks; a group whose largest brick fascicle
-    // table overflows halves its brick's largest dimension and the layout is
-    // rebuilt, until all groups fit (other groups keep their bricks).
-    const int B0 = std::max(2, ix->brick_dim);
-    const bool grouped = !ix->batch.vox_group.empty();
-    const int ngroups = grouped ? ix->batch.n : 1;
-    std::vector<BrickShape> shape(ngroups, BrickShape{B0, B0, B0});
-    for (int attempt = 0; attempt < 32 && !ok; ++attempt) {
-        assign_tiles(ix->nv, ijk, shape, ix->batch, H);
-        LIFE_TRY(upload(d_vox_tile, H.vox_tile, s));
-        LIFE_TRY(upload(d_vox_row, H.vox_row, s));
-        LIFE_TRY(upload(d_tile_brick, H.tile_brick, s));
-        const int bt = nbits64(H.n_tiles), bb = nbits64(H.n_bricks);
-        if (bt + 16 + bf > 64 || bb + bf > 64) {
-            set_error("tensor-core layout: sort key too wide");
-            return LIFE_ENOTSUP;
-        }
-        L.brick_fasc_ptr.release();
-        LIFE_TRY(L.brick_fasc_ptr.alloc(sizeof(int32_t) * (H.n_bricks + 1)));
-        if (m > 0) {
-            tile_key_kernel<<<grid1d(m), 256, 0, s>>>(ix->ukey.as<uint64_t>(), m, sa, sv, (1ull << ba) - 1,
-                                                      (1ull << bf) - 1, bf, d_vox_tile.as<int32_t>(),
-                                                      d_vox_row.as<int32_t>(), skey.as<uint64_t>(), spay.as<uint32_t>());
-            LIFE_CHECK_LAUNCH();
-            // from (v, a, f) order by a stable sort: a cell's entries keep their fascicle order
-            LIFE_TRY(radix_sort_pairs(skey, spay, m, bf, bt + 16 + bf, s));
-            brick_key_kernel<<<grid1d(m), 256, 0, s>>>(skey.as<uint64_t>(), m, bf, d_tile_brick.as<int32_t>(),
-                                                       key2.as<uint64_t>(), pay2.as<uint32_t>());
-            LIFE_CHECK_LAUNCH();
-            LIFE_TRY(radix_sort_pairs(key2, pay2, m, 0, bb + bf, s));
-            head_flag_kernel<<<grid1d(m), 256, 0, s>>>(key2.as<uint64_t>(), m, head.as<int32_t>());
-            LIFE_CHECK_LAUNCH();
-            LIFE_TRY(exclusive_scan_i32(head.as<int32_t>(), uidx.as<int32_t>(), m, s));
-            int32_t last[2];
-            LIFE_CUDA_TRY(cudaMemcpyAsync(&last[0], uidx.as<int32_t>() + m - 1, 4, cudaMemcpyDeviceToHost, s));
-            LIFE_CUDA_TRY(cudaMemcpyAsync(&last[1], head.as<int32_t>() + m - 1, 4, cudaMemcpyDeviceToHost, s));
-            LIFE_CUDA_TRY(cudaStreamSynchronize(s));
-            n_unique = last[0] + last[1];
-            L.brick_fasc.release();
-            LIFE_TRY(L.brick_fasc.alloc(sizeof(int32_t) * std::max(n_unique, 1)));
-            brick_fasc_kernel<<<grid1d(m), 256, 0, s>>>(key2.as<uint64_t>(), m, bf, head.as<int32_t>(),
-                                                        uidx.as<int32_t>(), (int32_t)H.n_bricks, n_unique,
-                                                        L.brick_fasc_ptr.as<int32_t>(), L.brick_fasc.as<int32_t>());
-            LIFE_CHECK_LAUNCH();
-        } else {
-            fill_kernel<<<1, 256, 0, s>>>(L.brick_fasc_ptr.as<int32_t>(), H.n_bricks + 1, 0);
-            LIFE_CHECK_LAUNCH();
-            LIFE_TRY(L.brick_fasc.alloc(sizeof(int32_t)));
-        }
-        hbptr.resize(H.n_bricks + 1);
-        LIFE_CUDA_TRY(cudaMemcpyAsync(hbptr.data(), L.brick_fasc_ptr.p, sizeof(int32_t) * hbptr.size(),
-                                      cudaMemcpyDeviceToHost, s));
-        LIFE_CUDA_TRY(cudaStreamSynchronize(s));
-        std::vector<int32_t> gmax(ngroups, 0);
-        int32_t mx = 0;
-        for (int64_t b = 0; b < H.n_bricks; ++b) {
-            const int32_t nfb = hbptr[b + 1] - hbptr[b];
-            const int g = grouped ? ix->batch.vox_group[H.tile_vox[(size_t)H.brick_tile_ptr[b] * TILE_V]] : 0;
-            gmax[g] = std::max(gmax[g], nfb);
-            mx = std::max(mx, nfb);
-        }
-        L.max_fb = mx;
-        ok = true;
-        bool shrunk = false;
-        for (int g = 0; g < ngroups; ++g) {
-            if (gmax[g] <= MAX_BRICK_FASC) continue;
-            ok = false;
-            BrickShape& sh = shape[g];
-            int* d = sh.x >= sh.y && sh.x >= sh.z ? &sh.x : (sh.y >= sh.z ? &sh.y : &sh.z);
-            if (*d > 1) {
-                *d = (*d + 1) / 2;
-                shrunk = true;
-            }
-        }
-        if (!ok && !shrunk) break;
-    }
-    {
-        const BrickShape& s0 = shape[0];
-        const bool cubic = s0.x == s0.y && s0.y == s0.z;
-        L.brick_edge = ijk.empty() ? 0 : (cubic ? s0.x : std::max(s0.x, std::max(s0.y, s0.z)));
-        L.brick_b = B0;
-    }
-    if (!ok) {
-        set_error("tensor-core layout: a brick touches %d fascicles (limit %d) even at the smallest brick",
-                  L.max_fb, MAX_BRICK_FASC);
-        return LIFE_ENOTSUP;
-    }
-    L.n_tiles = H.n_tiles;
-    L.n_bricks = H.n_bricks;
-    L.n_nnz = m;
-    {
-        // padded, 16-byte aligned per-brick weight slots for the DSC's bulk table loads
-        std::vector<int32_t> wptr(H.n_bricks + 1, 0);
-        for (int64_t b = 0; b < H.n_bricks; ++b) wptr[b + 1] = wptr[b] + (hbptr[b + 1] - hbptr[b] + 3) / 4 * 4;
-        L.wb_total = wptr[H.n_bricks];
-        L.n_brick_slots = hbptr[H.n_bricks];
-        LIFE_TRY(upload(L.wb_ptr, wptr, s));
-        LIFE_TRY(L.wb_src.alloc(sizeof(int32_t) * std::max<int64_t>(L.wb_total, 4)));
-        // gathered tables in global memory serve only the live-entry stream (the
-        // dense DSC gathers each brick's weights itself)
-        if (ix->sparse_dsc != 0 && ix->batch.vox_group.empty())
-            LIFE_TRY(L.wb.alloc(sizeof(float) * std::max<int64_t>(L.wb_total, 4)));
-        else
-            L.wb.release();
-        if (H.n_bricks > 0) {
-            wb_src_kernel<<<(unsigned)std::min<int64_t>(H.n_bricks, 65535), 128, 0, s>>>(
-                L.brick_fasc_ptr.as<int32_t>(), L.brick_fasc.as<int32_t>(), L.wb_ptr.as<int32_t>(),
-                (int32_t)H.n_bricks, L.wb_src.as<int32_t>());
-            LIFE_CHECK_LAUNCH();
-        }
-        LIFE_CUDA_TRY(cudaStreamSynchronize(s));  // wptr is a host temporary
-    }
-    if (!ix->batch.vox_group.empty()) {
-        // problem of each brick (every voxel of a brick belongs to one problem; row 0
-        // of a brick's first tile is always a voxel)
-        std::vector<int32_t> bp(H.n_bricks);
-        for (int64_t b = 0; b < H.n_bricks; ++b)
-            bp[b] = ix->batch.vox_group[H.tile_vox[(size_t)H.brick_tile_ptr[b] * TILE_V]];
-        LIFE_TRY(upload(ix->batch.brick_prob, bp, s));
-    }
-    const int n_c = L.kp / DKC;  // 128-atom chunks per tile
-    const int64_t n_segs = H.n_tiles * n_c;
-    // streams padded to whole 8-entry slots (the kernels load 16 bytes at a time)
-    const int64_t m_pad = (m + 7) / 8 * 8 + 8;
-    LIFE_TRY(L.va.alloc(sizeof(uint16_t) * m_pad));
-    LIFE_TRY(L.soff.alloc(sizeof(uint16_t) * m_pad));
-    LIFE_TRY(L.fl.alloc(sizeof(uint16_t) * m_pad));
-    LIFE_TRY(L.val.alloc((size_t)L.vbytes * m_pad));
-    LIFE_CUDA_TRY(cudaMemsetAsync(L.va.p, 0, sizeof(uint16_t) * m_pad, s));
-    LIFE_CUDA_TRY(cudaMemsetAsync(L.soff.p, 0, sizeof(uint16_t) * m_pad, s));
-    LIFE_CUDA_TRY(cudaMemsetAsync(L.fl.p, 0, sizeof(uint16_t) * m_pad, s));
-    LIFE_CUDA_TRY(cudaMemsetAsync(L.val.p, 0, (size_t)L.vbytes * m_pad, s));
-    LIFE_TRY(L.chunk_ptr.alloc(sizeof(int32_t) * (n_segs + 1)));
-    if (m > 0) {
-        local_fasc_kernel<<<grid1d(m), 256, 0, s>>>(key2.as<uint64_t>(), pay2.as<uint32_t>(), m, bf,
-                                                    head.as<int32_t>(), uidx.as<int32_t>(), L.brick_fasc_ptr.as<int32_t>(),
-                                                    L.fl.as<uint16_t>());
-        LIFE_CHECK_LAUNCH();
-        if (L.vbytes == 4)
-            tile_stream_kernel<<<grid1d(m), 256, 0, s>>>(skey.as<uint64_t>(), spay.as<uint32_t>(), m, bf,
-                                                         ix->uval.as<float>(), n_c, n_segs, L.va.as<uint16_t>(),
-                                                         L.soff.as<uint16_t>(), L.fl.as<uint16_t>(), L.val.as<float>(),
-                                                         L.chunk_ptr.as<int32_t>());
-        else
-            tile_stream_kernel<<<grid1d(m), 256, 0, s>>>(skey.as<uint64_t>(), spay.as<uint32_t>(), m, bf,
-                                                         ix->uval.as<float>(), n_c, n_segs, L.va.as<uint16_t>(),
-                                                         L.soff.as<uint16_t>(), L.fl.as<uint16_t>(),
-                                                         L.val.as<__nv_bfloat16>(), L.chunk_ptr.as<int32_t>());
-        LIFE_CHECK_LAUNCH();
-    } else {
-        fill_kernel<<<grid1d(n_segs + 1), 256, 0, s>>>(L.chunk_ptr.as<int32_t>(), n_segs + 1, 0);
-        LIFE_CHECK_LAUNCH();
-    }
-    L.run_vmax = 0.0f;
-    if (m > 0) {
-        TmpBuf rv;
-        LIFE_TRY(rv.alloc(sizeof(uint32_t), s));
-        LIFE_CUDA_TRY(cudaMemsetAsync(rv.p, 0, sizeof(uint32_t), s));
-        if (L.vbytes == 4)
-            run_vmax_kernel<<<grid1d(m), 256, 0, s>>>(L.soff.as<uint16_t>(), L.val.as<float>(), m, rv.as<uint32_t>());
-        else
-            run_vmax_kernel<<<grid1d(m), 256, 0, s>>>(L.soff.as<uint16_t>(), L.val.as<__nv_bfloat16>(), m,
-                                                      rv.as<uint32_t>());
-        LIFE_CHECK_LAUNCH();
-        uint32_t bits = 0u;
-        LIFE_CUDA_TRY(cudaMemcpyAsync(&bits, rv.p, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-        LIFE_CUDA_TRY(cudaStreamSynchronize(s));
-        std::memcpy(&L.run_vmax, &bits, sizeof(float));
-    }
-    LIFE_TRY(L.x_amax.alloc(sizeof(uint32_t) * (size_t)std::max(ix->num_sms, 1) * 8));
-    LIFE_CUDA_TRY(cudaMemsetAsync(L.x_amax.p, 0, sizeof(uint32_t) * (size_t)std::max(ix->num_sms, 1) * 8, s));
-    // WC streams (row quarter major inside each tile)
-    const int64_t n_wsegs = H.n_tiles * 4 * L.n_sub;
-    if (L.wc_stream) {
-        LIFE_TRY(L.wkey.alloc(sizeof(uint16_t) * m_pad));
-        LIFE_TRY(L.wfl.alloc(sizeof(uint16_t) * m_pad));
-        LIFE_TRY(L.wval.alloc((size_t)L.vbytes * m_pad));
-        LIFE_TRY(L.wseg_ptr.alloc(sizeof(int32_t) * (n_wsegs + 1)));
-        LIFE_CUDA_TRY(cudaMemsetAsync(L.wkey.p, 0, sizeof(uint16_t) * m_pad, s));
-        LIFE_CUDA_TRY(cudaMemsetAsync(L.wfl.p, 0, sizeof(uint16_t) * m_pad, s));
-        LIFE_CUDA_TRY(cudaMemsetAsync(L.wval.p, 0, (size_t)L.vbytes * m_pad, s));
-        if (m > 0) {
-            wc_key_kernel<<<grid1d(m), 256, 0, s>>>(skey.as<uint64_t>(), m, bf, key2.as<uint64_t>(), pay2.as<uint32_t>());
-            LIFE_CHECK_LAUNCH();
-            LIFE_TRY(radix_sort_pairs(key2, pay2, m, bf, nbits64(H.n_tiles) + 16 + bf, s));
-            if (L.vbytes == 4)
-                wc_stream_kernel<<<grid1d(m), 256, 0, s>>>(key2.as<uint64_t>(), pay2.as<uint32_t>(), m, bf,
-                                                           L.fl.as<uint16_t>(), L.val.as<float>(), L.n_sub, n_wsegs, 1,
-                                                           L.wkey.as<uint16_t>(), L.wfl.as<uint16_t>(),
-                                                           L.wval.as<float>(), L.wseg_ptr.as<int32_t>());
-            else
-                wc_stream_kernel<<<grid1d(m), 256, 0, s>>>(key2.as<uint64_t>(), pay2.as<uint32_t>(), m, bf,
-                                                           L.fl.as<uint16_t>(), L.val.as<__nv_bfloat16>(), L.n_sub,
-                                                           n_wsegs, 0, L.wkey.as<uint16_t>(), L.wfl.as<uint16_t>(),
-                                                           L.wval.as<__nv_bfloat16>(), L.wseg_ptr.as<int32_t>());
-            LIFE_CHECK_LAUNCH();
-        } else {
-            fill_kernel<<<grid1d(n_wsegs + 1), 256, 0, s>>>(L.wseg_ptr.as<int32_t>(), n_wsegs + 1, 0);
-            LIFE_CHECK_LAUNCH();
-        }
-    } else {
-        L.wkey.release();
-        L.wfl.release();
-        L.wval.release();
-        L.wseg_ptr.release();
-    }
-    LIFE_TRY(upload(L.tile_vox, H.tile_vox, s));
-    LIFE_TRY(upload(L.brick_tile_ptr, H.brick_tile_ptr, s));
-    // live-entry DSC stream: allocated at full size, filled on demand by a DSC call
-    L.sparse = ix->sparse_dsc != 0 && ix->batch.vox_group.empty();
-    if (L.sparse) {
-        LIFE_TRY(L.c_soff.alloc(sizeof(uint16_t) * m_pad));
-        LIFE_TRY(L.c_fl.alloc(sizeof(uint16_t) * m_pad));
-        LIFE_TRY(L.c_val.alloc(sizeof(__nv_bfloat16) * m_pad));
-        LIFE_CUDA_TRY(cudaMemsetAsync(L.c_soff.p, 0, sizeof(uint16_t) * m_pad, s));
-        LIFE_CUDA_TRY(cudaMemsetAsync(L.c_fl.p, 0, sizeof(uint16_t) * m_pad, s));
-        LIFE_CUDA_TRY(cudaMemsetAsync(L.c_val.p, 0, sizeof(__nv_bfloat16) * m_pad, s));
-        const int64_t n_chunks = std::max<int64_t>(H.n_tiles * (L.kp / 128), 1);
-        LIFE_TRY(L.c_chunk_end.alloc(sizeof(int32_t) * n_chunks));
-        LIFE_CUDA_TRY(cudaMemsetAsync(L.c_chunk_end.p, 0, sizeof(int32_t) * n_chunks, s));
-        LIFE_TRY(L.wb_live.alloc(std::max<int64_t>(L.wb_total, 4)));
-        LIFE_CUDA_TRY(cudaMemsetAsync(L.wb_live.p, 0, std::max<int64_t>(L.wb_total, 4), s));
-        LIFE_TRY(upload(L.tile_brick, H.tile_brick, s));
-        LIFE_TRY(L.sparse_ctl.alloc(sizeof(SparseCtl)));
-        LIFE_CUDA_TRY(cudaMemsetAsync(L.sparse_ctl.p, 0, sizeof(SparseCtl), s));
-    } else {
-        L.c_soff.release();
-        L.c_fl.release();
-        L.c_val.release();
-        L.c_chunk_end.release();
-        L.wb_live.release();
-        L.sparse_ctl.release();
-        L.tile_brick.release();
-    }
-    LIFE_TRY(L.brick_cv.alloc(sizeof(float) * std::max<int64_t>(H.n_bricks, 1)));
-    LIFE_TRY(L.tile_amax.alloc(sizeof(uint32_t) * 4 * std::max<int64_t>(H.n_tiles, 1)));
-    if (H.n_bricks > 0 && L.wc_stream && L.vbytes == 2) {  // the FP32 WC sums in FP32 tables
-        const int cv_smem = (int)sizeof(int32_t) * std::max(L.max_fb, 1);
-        LIFE_CUDA_TRY(cudaFuncSetAttribute(brick_cv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, cv_smem));
-        brick_cv_kernel<<<(unsigned)std::min<int64_t>(H.n_bricks, 65535), 256, cv_smem, s>>>(
-            L.brick_tile_ptr.as<int32_t>(), L.brick_fasc_ptr.as<int32_t>(), L.wseg_ptr.as<int32_t>(), 4 * L.n_sub,
-            L.wfl.as<uint16_t>(), L.wval.as<__nv_bfloat16>(), (int32_t)H.n_bricks, L.brick_cv.as<float>());
-        LIFE_CHECK_LAUNCH();
-    }
-    // largest bricks first
-    std::vector<int32_t> tptr(H.n_tiles + 1);
-    {
-        std::vector<int32_t> sp(n_segs + 1);
-        LIFE_CUDA_TRY(cudaMemcpyAsync(sp.data(), L.chunk_ptr.p, sizeof(int32_t) * sp.size(), cudaMemcpyDeviceToHost, s));
-        LIFE_CUDA_TRY(cudaStreamSynchronize(s));
-        for (int64_t t = 0; t <= H.n_tiles; ++t) tptr[t] = sp[t * n_c];
-    }
-    std::vector<int64_t> bnnz(H.n_bricks);
-    for (int64_t b = 0; b < H.n_bricks; ++b)
-        bnnz[b] = (int64_t)tptr[H.brick_tile_ptr[b + 1]] - tptr[H.brick_tile_ptr[b]] +
-                  64 * (H.brick_tile_ptr[b + 1] - H.brick_tile_ptr[b]);
-    std::vector<int32_t> order(H.n_bricks);
-    std::iota(order.begin(), order.end(), 0);
-    std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return bnnz[x] > bnnz[y]; });
-    LIFE_TRY(upload(L.brick_order, order, s));
-    LIFE_CUDA_TRY(cudaStreamSynchronize(s));
-    L.built = true;
-    return LIFE_OK;
-}
-
 __global__ void widen_bf16_kernel(const __nv_bfloat16* __restrict__ in, int64_t n, float* __restrict__ out) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         out[i] = __bfloat162float(in[i]);
@@ -950,6 +303,23 @@ __global__ void export_fl_kernel(const uint16_t* __restrict__ fl, const uint16_t
                                  uint16_t* __restrict__ out) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         out[i] = (uint16_t)((fl[i] >> 2) | (soff[i] & CONT));
+}
+
+// row | atom << 7 of each DSC-stream entry: the cell from its S byte offset, the
+// 128-atom chunk from the entry's place in chunk_ptr (n_seg chunks, n_c per tile).
+__global__ void export_va_kernel(const uint16_t* __restrict__ soff, const int32_t* __restrict__ chunk_ptr,
+                                 int64_t n_seg, int n_c, int64_t n, uint16_t* __restrict__ out) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        int64_t lo = 0, hi = n_seg - 1;  // the last chunk that starts at or before i
+        while (lo < hi) {
+            const int64_t mid = (lo + hi + 1) >> 1;
+            if (chunk_ptr[mid] <= i) lo = mid;
+            else hi = mid - 1;
+        }
+        const uint32_t so = soff[i] & 0x7FFFu;
+        const uint32_t row = (so >> 11) * 8 + ((so >> 4) & 7u), a = ((so >> 7) & 15u) * 8 + ((so >> 1) & 7u);
+        out[i] = (uint16_t)(row | ((a + (uint32_t)(lo % n_c) * DKC) << 7));
+    }
 }
 
 life_status export_tiles(life_index_s* ix, int32_t* tile_vox, int32_t* chunk_ptr, int32_t* brick_tile_ptr,
@@ -966,7 +336,11 @@ life_status export_tiles(life_index_s* ix, int32_t* tile_vox, int32_t* chunk_ptr
     LIFE_TRY(cp(brick_fasc_ptr, L.brick_fasc_ptr, sizeof(int32_t) * (L.n_bricks + 1)));
     LIFE_TRY(cp(brick_fasc, L.brick_fasc, L.brick_fasc.bytes));
     LIFE_TRY(cp(brick_order, L.brick_order, sizeof(int32_t) * L.n_bricks));
-    LIFE_TRY(cp(va, L.va, sizeof(uint16_t) * L.n_nnz));
+    if (va && L.n_nnz > 0) {
+        export_va_kernel<<<grid1d(L.n_nnz), 256, 0, s>>>(L.soff.as<uint16_t>(), L.chunk_ptr.as<int32_t>(),
+                                                         L.n_tiles * (L.kp / DKC), L.kp / DKC, L.n_nnz, va);
+        LIFE_CHECK_LAUNCH();
+    }
     if (fl && L.n_nnz > 0) {
         export_fl_kernel<<<grid1d(L.n_nnz), 256, 0, s>>>(L.fl.as<uint16_t>(), L.soff.as<uint16_t>(), L.n_nnz, fl);
         LIFE_CHECK_LAUNCH();
@@ -992,7 +366,6 @@ struct TcArgs {
     const int32_t* brick_fasc_ptr;
     const int32_t* brick_fasc;
     const int32_t* brick_order;
-    const uint16_t* va;
     const uint16_t* soff;
     const uint16_t* fl;
     const __nv_bfloat16* val;
@@ -2797,7 +2170,6 @@ static TcArgs make_args(life_index_s* ix) {
     A.brick_fasc_ptr = L.brick_fasc_ptr.as<int32_t>();
     A.brick_fasc = L.brick_fasc.as<int32_t>();
     A.brick_order = L.brick_order.as<int32_t>();
-    A.va = L.va.as<uint16_t>();
     A.soff = L.soff.as<uint16_t>();
     A.wkey = L.wkey.as<uint16_t>();
     A.wfl = L.wfl.as<uint16_t>();

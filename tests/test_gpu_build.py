@@ -55,3 +55,32 @@ def test_unaligned_input_arrays(life):
     ref = oracle.canon(a, v, f, x, 50, 300, 700)
     got = [y.cpu().numpy() for y in life.life_index_export(idx)]
     assert all(np.array_equal(g, r) for g, r in zip(got, (ref.atom, ref.voxel, ref.fasc, ref.val)))
+
+
+# one voxel-id brick and several; a fascicle range of more than one bitmap window
+# (2^19 ids); Na = 512 (four chunks); a tile of more entries a pass than are staged at
+# once (19456); single-entry and empty voxels
+@pytest.mark.parametrize("precision", ["bf16", "fp32"])
+@pytest.mark.parametrize("dims", [(360, 700, 3000, 60000), (129, 1025, 600000, 30000), (512, 300, 2000, 40000),
+                                  (20, 60, 9000, 90000), (384, 127, 4000, 1), (1, 640, 15000, 20000)])
+def test_tile_layout_bit_exact(life, dims, precision):
+    from test_gpu_tc import expected_tiles
+    na, nv, nf, n = dims
+    if precision == "fp32" and na > 384:
+        pytest.skip("FP32 storage on the tensor cores needs Na <= 384")
+    a, v, f, x = raw_list(n, na, nv, nf, n + nv, False)
+    v[n // 3:n // 2] = nv // 2        # one very full voxel
+    prec = life.LIFE_BF16 if precision == "bf16" else life.LIFE_FP32
+    idx = life.index_from_arrays(a, v, f, x, 16, na, nv, nf, precision=prec, algo=life.LIFE_ALGO_TC, brick_dim=6)
+    phi = oracle.canon(a, v, f, x, na, nv, nf)
+    info, m = idx.info(), idx.nnz
+    got = {k: t.cpu().numpy() for k, t in life.life_index_export_tiles(idx).items()}
+    exp = expected_tiles(phi, got["tile_vox"], got["brick_tile_ptr"], nv, info["n_sub"])
+    for k in ("chunk_ptr", "brick_fasc_ptr"):
+        assert np.array_equal(got[k], exp[k]), k
+    assert np.array_equal(got["va"][:m].view(np.uint16), exp["va"])
+    assert np.array_equal(got["fl"][:m].view(np.uint16), exp["fl"])
+    assert np.array_equal(got["brick_fasc"][:info["n_brick_fasc"]], exp["brick_fasc"])
+    val = got["val"][:m] if precision == "bf16" else torch.from_numpy(got["val"][:m]).bfloat16().float().numpy()
+    assert np.array_equal(val, exp["val"])
+    assert np.array_equal(np.sort(got["tile_vox"][got["tile_vox"] >= 0]), np.arange(nv))
