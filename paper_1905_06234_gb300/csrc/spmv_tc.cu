@@ -1439,6 +1439,69 @@ __global__ void __launch_bounds__(AMAX_THREADS) wc_amax_kernel(TcArgs A) {
     }
 }
 
+// The loader warps take a tile of r in units of 8 values of θ of one row: thread lt
+// takes units lt, lt + WC_LOAD_THREADS, ... in batches of UB, each batch's loads
+// issued together.  ngrp = np / 8 units a row; unit / ngrp by a multiplication
+// (units < 4096, ngrp <= 16: exact).
+struct RUnits {
+    int ngrp;
+    uint32_t magic;
+    __device__ __forceinline__ explicit RUnits(int np) : ngrp(np / 8), magic((65536u + np / 8 - 1) / (np / 8)) {}
+    __device__ __forceinline__ int row(int u) const { return (int)(((uint32_t)u * magic) >> 16); }
+};
+
+// The voxels (-1 for none) of the rows of this thread's UB units from unit u0 on.
+template <int UB>
+__device__ __forceinline__ void load_r_voxels(const TcArgs& A, int t, int u0, const RUnits& R, int (&v)[UB]) {
+#pragma unroll
+    for (int s = 0; s < UB; ++s) {
+        const int row = R.row(u0 + s * WC_LOAD_THREADS);
+        v[s] = row < TILE_V ? __ldg(A.tile_vox + (int64_t)t * TILE_V + row) : -1;
+    }
+}
+
+// Loads one tile of r for the loader warps and hands each unit to emit(row, θ / 8,
+// values).  v holds the voxels of the first batch on entry; each later batch's are
+// read while the batch before it is on its way, so that a batch costs one round
+// trip to memory, not two.  (Looked up before each unit's load, they made a tile of
+// the medium workload 9 us of loading, in a kernel that needs 6 us a tile for the
+// rest.  Handed out by shuffles from a register of each lane they did worse at the
+// paper's density: the scatter warps keep the shuffles' pipe busy.)
+template <int UB, class Emit>
+__device__ __forceinline__ void load_r_tile(const TcArgs& A, int t, const RUnits& R, int (&v)[UB], int lt, bool vec,
+                                            Emit emit) {
+    const int total = TILE_V * R.ngrp;
+    for (int u0 = lt; u0 < total; u0 += UB * WC_LOAD_THREADS) {
+        float4 lo[UB], hi[UB];
+#pragma unroll
+        for (int s = 0; s < UB; ++s) {
+            const int u = u0 + s * WC_LOAD_THREADS, g = u - R.row(u) * R.ngrp;
+            const float* src = A.x + (int64_t)A.nt * v[s] + 8 * g;
+            const int n = v[s] >= 0 ? A.nt - 8 * g : 0;  // values of this unit inside the row
+            lo[s] = hi[s] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (vec) {
+                if (n >= 4) lo[s] = __ldg(reinterpret_cast<const float4*>(src));
+                if (n >= 8) hi[s] = __ldg(reinterpret_cast<const float4*>(src) + 1);
+            } else {
+                if (n > 0) lo[s].x = __ldg(src);
+                if (n > 1) lo[s].y = __ldg(src + 1);
+                if (n > 2) lo[s].z = __ldg(src + 2);
+                if (n > 3) lo[s].w = __ldg(src + 3);
+                if (n > 4) hi[s].x = __ldg(src + 4);
+                if (n > 5) hi[s].y = __ldg(src + 5);
+                if (n > 6) hi[s].z = __ldg(src + 6);
+                if (n > 7) hi[s].w = __ldg(src + 7);
+            }
+        }
+        load_r_voxels(A, t, u0 + UB * WC_LOAD_THREADS, R, v);
+#pragma unroll
+        for (int s = 0; s < UB; ++s) {
+            const int u = u0 + s * WC_LOAD_THREADS, row = R.row(u);
+            if (u < total) emit(row, u - row * R.ngrp, lo[s], hi[s]);
+        }
+    }
+}
+
 __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ uint64_t r_full[2], r_empty[2], z_full[ZSLOTS], z_empty[ZSLOTS], fin_bar;
@@ -1643,8 +1706,9 @@ __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
         // ---------------- R tile loader: r[:, v] -> FP16 A operand times 2^kR of the
         // brick (rows = voxels, K = θ); kR from the brick's max |r|, as the scatter warps compute it
         const int lt = tid - WC_SCAT_THREADS;
-        const int ngrp = A.np / 8;
-        const bool vec = A.vec4 != 0 && (A.nt % 8) == 0;
+        const bool vec = A.vec4 != 0;
+        const RUnits RU(A.np);
+        int vv[4], tv = -1;  // the first batch's voxels of tile tv
         uint32_t tcount = 0;
         bool stop = false;
         for (int r = 0; !stop; ++r) {
@@ -1660,58 +1724,28 @@ __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
                 // R buffer rb, used for the k-th time (tiles go round the buffers)
                 const uint32_t rb = A.rbufs == 2 ? (tcount & 1u) : 0u, rk = A.rbufs == 2 ? (tcount >> 1) : tcount;
                 unsigned char* Rb = Rs + rb * r_bytes;
+                if (tv != t) load_r_voxels(A, t, lt, RU, vv);
                 if (!warp_wait(&r_empty[rb], (rk & 1u) ^ 1u, &abort_flag)) {
                     abort_flag = 1;
                     stop = true;
                     break;
                 }
-                const int total = TILE_V * ngrp;
-                for (int u0 = lt; u0 < total; u0 += 4 * WC_LOAD_THREADS) {
-                    float4 lo[4], hi[4];
-#pragma unroll
-                    for (int s = 0; s < 4; ++s) {
-                        const int u = u0 + s * WC_LOAD_THREADS;
-                        lo[s] = make_float4(0.f, 0.f, 0.f, 0.f);
-                        hi[s] = lo[s];
-                        if (u < total) {
-                            const int row = u / ngrp, g8 = u % ngrp;
-                            const int v = A.tile_vox[(int64_t)t * TILE_V + row];
-                            if (v >= 0) {
-                                const float* src = A.x + (int64_t)A.nt * v + 8 * g8;
-                                if (vec && 8 * g8 + 8 <= A.nt) {
-                                    lo[s] = __ldg(reinterpret_cast<const float4*>(src));
-                                    hi[s] = __ldg(reinterpret_cast<const float4*>(src) + 1);
-                                } else {
-                                    float e[8];
-#pragma unroll
-                                    for (int z = 0; z < 8; ++z) e[z] = (8 * g8 + z < A.nt) ? src[z] : 0.0f;
-                                    lo[s] = make_float4(e[0], e[1], e[2], e[3]);
-                                    hi[s] = make_float4(e[4], e[5], e[6], e[7]);
-                                }
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int s = 0; s < 4; ++s) {
-                        const int u = u0 + s * WC_LOAD_THREADS;
-                        if (u >= total) continue;
-                        const int row = u / ngrp, g8 = u % ngrp;
-                        __half2 p0 = __floats2half2_rn(lo[s].x * rs, lo[s].y * rs);
-                        __half2 p1 = __floats2half2_rn(lo[s].z * rs, lo[s].w * rs);
-                        __half2 p2 = __floats2half2_rn(hi[s].x * rs, hi[s].y * rs);
-                        __half2 p3 = __floats2half2_rn(hi[s].z * rs, hi[s].w * rs);
-                        uint4 pk;
-                        pk.x = *reinterpret_cast<uint32_t*>(&p0);
-                        pk.y = *reinterpret_cast<uint32_t*>(&p1);
-                        pk.z = *reinterpret_cast<uint32_t*>(&p2);
-                        pk.w = *reinterpret_cast<uint32_t*>(&p3);
-                        *reinterpret_cast<uint4*>(Rb + kmajor_off(row, 8 * g8, SBO_K)) = pk;
-                    }
-                }
+                load_r_tile(A, t, RU, vv, lt, vec, [&](int row, int g8, const float4& lo, const float4& hi) {
+                    const __half2 p0 = __floats2half2_rn(lo.x * rs, lo.y * rs), p1 = __floats2half2_rn(lo.z * rs, lo.w * rs);
+                    const __half2 p2 = __floats2half2_rn(hi.x * rs, hi.y * rs), p3 = __floats2half2_rn(hi.z * rs, hi.w * rs);
+                    uint4 pk;
+                    pk.x = *reinterpret_cast<const uint32_t*>(&p0);
+                    pk.y = *reinterpret_cast<const uint32_t*>(&p1);
+                    pk.z = *reinterpret_cast<const uint32_t*>(&p2);
+                    pk.w = *reinterpret_cast<const uint32_t*>(&p3);
+                    *reinterpret_cast<uint4*>(Rb + kmajor_off(row, 8 * g8, SBO_K)) = pk;
+                });
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&r_full[rb]);
                 ++tcount;
+                tv = t + 1 < A.brick_tile_ptr[brick + 1] ? t + 1 : next_brick >= 0 ? A.brick_tile_ptr[next_brick] : t;
+                load_r_voxels(A, tv, lt, RU, vv);  // of the tile after this one
                 // pull the voxel rows of r of the tile A.rbufs ahead into L2 (the
                 // loader runs A.rbufs - 1 tiles ahead of the tensor cores), so that
                 // loading it later is not a chain of DRAM round trips
@@ -1991,8 +2025,9 @@ __global__ void __maxnreg__(96) wc_tc32_kernel(TcArgs A) {
         // ---------------- R tile loader: r[:, v]·2^kR of the brick as FP16 hi and lo
         // parts (rows = voxels, K = θ), kR as the scatter warps compute it
         const int lt = tid - WC_SCAT_THREADS;
-        const int ngrp = A.np / 8;
-        const bool vec = A.vec4 != 0 && (A.nt % 8) == 0;
+        const bool vec = A.vec4 != 0;
+        const RUnits RU(A.np);
+        int vv[2], tv = -1;  // the first batch's voxels of tile tv
         uint32_t tcount = 0;
         bool stop = false;
         for (int r = 0; !stop; ++r) {
@@ -2007,56 +2042,28 @@ __global__ void __maxnreg__(96) wc_tc32_kernel(TcArgs A) {
             for (int t = A.brick_tile_ptr[brick]; t < A.brick_tile_ptr[brick + 1]; ++t) {
                 const uint32_t rb = A.rbufs == 2 ? (tcount & 1u) : 0u, rk = A.rbufs == 2 ? (tcount >> 1) : tcount;
                 unsigned char* Rb = Rs + rb * r_bytes;
+                if (tv != t) load_r_voxels(A, t, lt, RU, vv);
                 if (!warp_wait(&r_empty[rb], (rk & 1u) ^ 1u, &abort_flag)) {
                     abort_flag = 1;
                     stop = true;
                     break;
                 }
-                const int total = TILE_V * ngrp;
-                for (int u0 = lt; u0 < total; u0 += 2 * WC_LOAD_THREADS) {
-                    float4 lo[2], hi[2];
-#pragma unroll
-                    for (int s2 = 0; s2 < 2; ++s2) {
-                        const int u = u0 + s2 * WC_LOAD_THREADS;
-                        lo[s2] = make_float4(0.f, 0.f, 0.f, 0.f);
-                        hi[s2] = lo[s2];
-                        if (u < total) {
-                            const int row = u / ngrp, g8 = u % ngrp;
-                            const int v = A.tile_vox[(int64_t)t * TILE_V + row];
-                            if (v >= 0) {
-                                const float* src = A.x + (int64_t)A.nt * v + 8 * g8;
-                                if (vec && 8 * g8 + 8 <= A.nt) {
-                                    lo[s2] = __ldg(reinterpret_cast<const float4*>(src));
-                                    hi[s2] = __ldg(reinterpret_cast<const float4*>(src) + 1);
-                                } else {
-                                    float e[8];
-#pragma unroll
-                                    for (int z = 0; z < 8; ++z) e[z] = (8 * g8 + z < A.nt) ? src[z] : 0.0f;
-                                    lo[s2] = make_float4(e[0], e[1], e[2], e[3]);
-                                    hi[s2] = make_float4(e[4], e[5], e[6], e[7]);
-                                }
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int s2 = 0; s2 < 2; ++s2) {
-                        const int u = u0 + s2 * WC_LOAD_THREADS;
-                        if (u >= total) continue;
-                        const int row = u / ngrp, g8 = u % ngrp;
-                        uint4 ph, pl;
-                        split_f16x2(lo[s2].x * rs, lo[s2].y * rs, ph.x, pl.x);
-                        split_f16x2(lo[s2].z * rs, lo[s2].w * rs, ph.y, pl.y);
-                        split_f16x2(hi[s2].x * rs, hi[s2].y * rs, ph.z, pl.z);
-                        split_f16x2(hi[s2].z * rs, hi[s2].w * rs, ph.w, pl.w);
-                        const uint32_t off = kmajor_off(row, 8 * g8, SBO_K);
-                        *reinterpret_cast<uint4*>(Rb + off) = ph;
-                        *reinterpret_cast<uint4*>(Rb + r_part + off) = pl;
-                    }
-                }
+                load_r_tile(A, t, RU, vv, lt, vec, [&](int row, int g8, const float4& lo, const float4& hi) {
+                    uint4 ph, pl;
+                    split_f16x2(lo.x * rs, lo.y * rs, ph.x, pl.x);
+                    split_f16x2(lo.z * rs, lo.w * rs, ph.y, pl.y);
+                    split_f16x2(hi.x * rs, hi.y * rs, ph.z, pl.z);
+                    split_f16x2(hi.z * rs, hi.w * rs, ph.w, pl.w);
+                    const uint32_t off = kmajor_off(row, 8 * g8, SBO_K);
+                    *reinterpret_cast<uint4*>(Rb + off) = ph;
+                    *reinterpret_cast<uint4*>(Rb + r_part + off) = pl;
+                });
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&r_full[rb]);
                 ++tcount;
+                tv = t + 1 < A.brick_tile_ptr[brick + 1] ? t + 1 : next_brick >= 0 ? A.brick_tile_ptr[next_brick] : t;
+                load_r_voxels(A, tv, lt, RU, vv);  // of the tile after this one
                 // pull the voxel rows of r of the tile A.rbufs ahead into L2
                 int tn = t + A.rbufs;
                 if (tn >= A.brick_tile_ptr[brick + 1]) {
