@@ -37,8 +37,6 @@ namespace life {
 
 life_status export_layout(life_index_s* ix, int layout, int32_t* atom, int32_t* voxel, int32_t* fasc, float* val,
                           cudaStream_t s);
-life_status dsc_tc(life_index_s* ix, const float* D, const float* w, const float* b, float* y, double* partial,
-                   int* n_partial, const life_sbb_state* gate, int gate_mode, cudaStream_t s, const BatchGate& bg);
 life_status build_tile_layout(life_index_s* ix, cudaStream_t s);
 
 __global__ void offset_ids_kernel(int32_t* __restrict__ voxel, int32_t* __restrict__ fasc, int64_t m, int32_t voff,

@@ -49,8 +49,8 @@ static bool use_tc(const life_index_s* ix) { return ix->algo == LIFE_ALGO_TC && 
 
 life_status spmv_dsc(life_index_s* ix, const float* D, const float* w, const float* b, float* y, double* partial,
                      int* n_partial, const life_sbb_state* gate, int gate_mode, cudaStream_t s,
-                     const BatchGate& bg) {
-    if (use_tc(ix)) return dsc_tc(ix, D, w, b, y, partial, n_partial, gate, gate_mode, s, bg);
+                     const BatchGate& bg, float* zero) {
+    if (use_tc(ix)) return dsc_tc(ix, D, w, b, y, partial, n_partial, gate, gate_mode, s, bg, zero);
     return dsc_simt(ix, D, w, b, y, partial, n_partial, gate, gate_mode, s, bg);
 }
 
@@ -61,6 +61,8 @@ __global__ void zero_f32_kernel(float* __restrict__ x, int64_t n) {
 
 life_status spmv_wc(life_index_s* ix, const float* D, const float* r, float* g, const life_sbb_state* gate,
                     int gate_mode, cudaStream_t s, const BatchGate& bg, bool r_is_dsc_out) {
+    // an FP32-storage TC index may run its DSC on the tensor cores and its WC on the CUDA cores
+    if (use_tc(ix) && ix->tile.wc_stream) return wc_tc(ix, D, r, g, gate, gate_mode, s, bg, r_is_dsc_out);
     if (bg.live) {
         // a kernel rather than a memset, so the batched step is all kernel nodes
         zero_f32_kernel<<<ix->num_sms * 2, 256, 0, s>>>(g, ix->nf);
@@ -68,8 +70,6 @@ life_status spmv_wc(life_index_s* ix, const float* D, const float* r, float* g, 
     } else {
         LIFE_CUDA_TRY(cudaMemsetAsync(g, 0, sizeof(float) * (size_t)ix->nf, s));
     }
-    // an FP32-storage TC index runs its DSC on the tensor cores and its WC on the CUDA cores
-    if (use_tc(ix) && ix->tile.wc_stream) return wc_tc(ix, D, r, g, gate, gate_mode, s, bg, r_is_dsc_out);
     return wc_simt(ix, D, r, g, gate, gate_mode, s, bg);
 }
 
@@ -240,7 +240,8 @@ extern "C" life_status life_index_get_info(life_index idx, life_index_info* out)
                             &idx->tile.wfl, &idx->tile.wval, &idx->tile.wseg_ptr, &idx->tile.wb_src,
                             &idx->tile.wb_ptr, &idx->tile.wb, &idx->tile.brick_cv, &idx->tile.tile_amax, &idx->red,
                             &idx->tile.c_soff, &idx->tile.c_fl, &idx->tile.c_val, &idx->tile.c_chunk_end,
-                            &idx->tile.wb_live, &idx->tile.sparse_ctl, &idx->tile.tile_brick, &idx->tile.x_amax};
+                            &idx->tile.wb_live, &idx->tile.sparse_ctl, &idx->tile.tile_brick, &idx->tile.x_amax, &idx->tile.d_img,
+                            &idx->tile.d_info};
     int64_t tot = 0;
     for (auto* b : bufs) tot += (int64_t)b->bytes;
     I.device_bytes = tot;

@@ -188,6 +188,9 @@ struct TileLayout {
     DevBuf tile_brick;       // int32 [n_tiles] brick of each tile
     float run_vmax = 0.0f;   // largest Σ|val| (BF16 values) over one (atom, voxel) run of the DSC stream
     DevBuf x_amax;           // uint32 [num_sms·8] bits of max |x| per block of a DSC's weight gather
+    DevBuf d_img;            // BF16 storage: the current call's D as FP16 MMA operands, np x kp for the DSC
+                             // (rows θ), then for the WC (rows = atoms)
+    DevBuf d_info;           // uint32: their scale exponent, then column-sum maxima of |D| per block of atoms
     DevBuf brick_cv;         // float [n_bricks]: (largest entry count of a fascicle) x (largest |val|)
     DevBuf tile_amax;        // uint32 [n_tiles * 4]: bits of |r| maxima, four slots per tile whose
                              // maximum is the tile's max |r| (per row quarter from the BF16 DSC, per
@@ -288,17 +291,19 @@ int simt_total_warps(const life_index_s* ix);
 // -------------------------------------------------------------- TC SpMVs
 life_status dsc_tc(life_index_s* ix, const float* D, const float* w, const float* b, float* y,
                    double* partial, int* n_partial, const life_sbb_state* gate, int gate_mode,
-                   cudaStream_t s, const BatchGate& bg = BatchGate());
-// r_is_dsc_out: r is the y that the last tensor-core DSC on this index wrote, so its
-// per-tile max |r| (written by that DSC's epilogue) is already in place.
+                   cudaStream_t s, const BatchGate& bg = BatchGate(), float* zero = nullptr);
+// r_is_dsc_out: r is the y that the last tensor-core DSC on this index wrote, with the
+// same D and with zero = g, so its per-tile max |r| (written by that DSC's epilogue),
+// D's operands and the zeroed g are already in place.
 life_status wc_tc(life_index_s* ix, const float* D, const float* r, float* g, const life_sbb_state* gate,
                   int gate_mode, cudaStream_t s, const BatchGate& bg = BatchGate(), bool r_is_dsc_out = false);
 
 // ------------------------------------------------------------- dispatch
-// DSC / WC on whichever kernels the index uses (WC zeroes g first).
+// DSC / WC on whichever kernels the index uses (WC zeroes g first).  zero: the g of a
+// WC that follows with r_is_dsc_out = true, cleared by the tensor-core DSC's launches.
 life_status spmv_dsc(life_index_s* ix, const float* D, const float* w, const float* b, float* y, double* partial,
                      int* n_partial, const life_sbb_state* gate, int gate_mode, cudaStream_t s,
-                     const BatchGate& bg = BatchGate());
+                     const BatchGate& bg = BatchGate(), float* zero = nullptr);
 life_status spmv_wc(life_index_s* ix, const float* D, const float* r, float* g, const life_sbb_state* gate,
                     int gate_mode, cudaStream_t s, const BatchGate& bg = BatchGate(), bool r_is_dsc_out = false);
 life_status build_index_layouts(life_index_s* ix, const int32_t* atom, const int32_t* voxel, const int32_t* fasc,

@@ -328,7 +328,7 @@ life_status sbb_enqueue_step(life_index_s* ix, const float* D, const float* b, f
     const int vgrid = std::min(device_sm_count() * 4, RED_SLOTS);
     int ne = 0, nv_ = 0, nu = 0;
     // e = M w − b, Σ e²
-    LIFE_TRY(spmv_dsc(ix, D, w, b, W.e, W.pe, &ne, st, GATE_ACTIVE, s));
+    LIFE_TRY(spmv_dsc(ix, D, w, b, W.e, W.pe, &ne, st, GATE_ACTIVE, s, BatchGate(), W.g));
     // g = M^T e
     LIFE_TRY(spmv_wc(ix, D, W.e, W.g, st, GATE_ACTIVE, s, BatchGate(), true));
     // g~, Σ g~²
@@ -337,7 +337,7 @@ life_status sbb_enqueue_step(life_index_s* ix, const float* D, const float* b, f
     sbb_scalars1_kernel<<<1, RED_THREADS, 0, s>>>(st, W.pe, ne, W.pg, vgrid, tol, eq7_on_even);
     LIFE_CHECK_LAUNCH();
     // v' = M g~ (stored only on Eq. 8 iterations), Σ v'²
-    LIFE_TRY(spmv_dsc(ix, D, W.gt, nullptr, W.e, W.pv, &nv_, st, 3, s));
+    LIFE_TRY(spmv_dsc(ix, D, W.gt, nullptr, W.e, W.pv, &nv_, st, GATE_ACTIVE_Y_EQ8, s, BatchGate(), W.u));
     // v'' = M^T v', Σ v''² (Eq. 8 iterations only)
     LIFE_TRY(spmv_wc(ix, D, W.e, W.u, st, GATE_EQ8, s, BatchGate(), true));
     LIFE_TRY(sumsq_f32(W.u, nf, W.pu, &nu, st, GATE_EQ8, s));
@@ -369,7 +369,7 @@ life_status sbb_enqueue_shard_phase(life_index_s* ix, const float* D, const floa
     const int vgrid = std::min(device_sm_count() * 4, RED_SLOTS);
     if (phase == 1) {
         int ne = 0;
-        LIFE_TRY(spmv_dsc(ix, D, w, b, W.e, W.pe, &ne, st, GATE_ACTIVE, s));
+        LIFE_TRY(spmv_dsc(ix, D, w, b, W.e, W.pe, &ne, st, GATE_ACTIVE, s, BatchGate(), g));
         LIFE_TRY(reduce_partials(W.pe, ne, scal, s));
         LIFE_TRY(spmv_wc(ix, D, W.e, g, st, GATE_ACTIVE, s, BatchGate(), true));
     } else if (phase == 2) {
@@ -378,7 +378,7 @@ life_status sbb_enqueue_shard_phase(life_index_s* ix, const float* D, const floa
         LIFE_CHECK_LAUNCH();
         sbb_scalars1_kernel<<<1, RED_THREADS, 0, s>>>(st, scal, 1, W.pg, vgrid, tol, eq7_on_even);
         LIFE_CHECK_LAUNCH();
-        LIFE_TRY(spmv_dsc(ix, D, W.gt, nullptr, W.e, W.pv, &nv_, st, GATE_ACTIVE_Y_EQ8, s));
+        LIFE_TRY(spmv_dsc(ix, D, W.gt, nullptr, W.e, W.pv, &nv_, st, GATE_ACTIVE_Y_EQ8, s, BatchGate(), u));
         LIFE_TRY(reduce_partials(W.pv, nv_, scal + 1, s));
         LIFE_TRY(spmv_wc(ix, D, W.e, u, st, GATE_EQ8, s, BatchGate(), true));
     } else {
@@ -556,7 +556,7 @@ life_status sbb_enqueue_batch_step(life_index_s* ix, const float* D, life_sbb_st
     batch_live_kernel<<<1, RED_THREADS, 0, s>>>(n, st, W.live);
     LIFE_CHECK_LAUNCH();
     // e = M w − b, Σ e² per problem
-    LIFE_TRY(spmv_dsc(ix, D, W.w, W.b, W.e, W.pe, nullptr, st, GATE_ACTIVE, s, bg));
+    LIFE_TRY(spmv_dsc(ix, D, W.w, W.b, W.e, W.pe, nullptr, st, GATE_ACTIVE, s, bg, W.g));
     // g = M^T e
     LIFE_TRY(spmv_wc(ix, D, W.e, W.g, st, GATE_ACTIVE, s, bg, true));
     batch_project_kernel<<<vgrid, RED_THREADS, 0, s>>>(W.w, W.g, W.gt, fasc_off, W.pg, W.live);
@@ -564,7 +564,7 @@ life_status sbb_enqueue_batch_step(life_index_s* ix, const float* D, life_sbb_st
     batch_scalars1_kernel<<<n, RED_THREADS, 0, s>>>(st, W.live, W.pe, part_off, W.pg, BATCH_VGX, tol, eq7_on_even);
     LIFE_CHECK_LAUNCH();
     // v' = M g~ (stored on Eq. 8 iterations), Σ v'²
-    LIFE_TRY(spmv_dsc(ix, D, W.gt, nullptr, W.e, W.pv, nullptr, st, GATE_ACTIVE_Y_EQ8, s, bg));
+    LIFE_TRY(spmv_dsc(ix, D, W.gt, nullptr, W.e, W.pv, nullptr, st, GATE_ACTIVE_Y_EQ8, s, bg, W.u));
     // v'' = M^T v', Σ v''² (Eq. 8 iterations)
     LIFE_TRY(spmv_wc(ix, D, W.e, W.u, st, GATE_EQ8, s, bg, true));
     batch_sumsq_kernel<<<vgrid, RED_THREADS, 0, s>>>(W.u, fasc_off, W.pu, W.live, st);

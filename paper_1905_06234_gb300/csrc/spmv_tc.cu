@@ -1,4 +1,4 @@
-// Tensor-core (tcgen05) SpMVs on the brick/tile layout, BF16 storage.
+// Tensor-core (tcgen05) SpMVs on the brick/tile layout.
 //
 // Both SpMVs are split into a sparse part and a dense contraction with the
 // dictionary (Eq. 3: M_v = D Phi_v):
@@ -42,7 +42,7 @@ __device__ __forceinline__ uint32_t absmax4_bits(const float4& v) {
 }
 
 // Block maximum of the bits of |x| (non-negative floats order as unsigned ints,
-// NaN above +inf), written by thread 0 to out[blockIdx.x].
+// NaN above +inf), written by thread 0 to *out.
 __device__ __forceinline__ void block_absmax_out(uint32_t m, uint32_t* out) {
     __shared__ uint32_t wmax[32];
     for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -51,22 +51,8 @@ __device__ __forceinline__ void block_absmax_out(uint32_t m, uint32_t* out) {
     if (threadIdx.x == 0) {
         uint32_t t = 0u;
         for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t = max(t, wmax[i]);
-        out[blockIdx.x] = t;
+        *out = t;
     }
-}
-
-// Per block, the bits of max |x| over the finite values of x: the scale of the
-// DSC's FP16 S operand when the DSC gathers each brick's weights itself.  (A NaN
-// or inf weight makes its run sums non-finite whatever the scale; leaving it out
-// keeps every other S value scaled into FP16's range.)  One block per SM.
-__global__ void __launch_bounds__(256) x_amax_kernel(const float* __restrict__ x, int64_t n,
-                                                     uint32_t* __restrict__ amax) {
-    uint32_t m = 0u;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t bits = __float_as_uint(__ldg(x + i)) & 0x7FFFFFFFu;
-        if (bits < 0x7F800000u) m = max(m, bits);
-    }
-    block_absmax_out(m, amax);
 }
 
 // ------------------------------------------------- live-entry DSC stream
@@ -179,7 +165,7 @@ __global__ void __launch_bounds__(GATHER_THREADS, 8) wb_gather_live_kernel(const
         atomicAdd(&blk_n, cnt);
         atomicOr(&blk_stale, stale);
     }
-    block_absmax_out(am, amax);   // (its barrier also orders the block counts above)
+    block_absmax_out(am, amax + blockIdx.x);   // (its barrier also orders the block counts above)
     if (threadIdx.x == 0) {
         if (blk_n) atomicAdd(&ctl->n_live, (unsigned long long)blk_n);
         if (blk_stale) atomicOr(&ctl->stale, 1u);
@@ -388,7 +374,10 @@ struct TcArgs {
     uint32_t* tile_amax;      // bits of |r| maxima, 4 slots per tile (their max is the tile's): DSC writes, WC reads
     const life_sbb_state* gate;
     int gate_mode;
-    const uint32_t* x_amax;    // DSC: bits of max |x| per block of this call's weight gather
+    const unsigned char* d_img;  // BF16 storage: D as this kernel's FP16 MMA operand (np x kp, K-major)
+    const uint32_t* d_info;      // [0] kD, the operand's scale exponent; [1 ..] column sums of |D| (n_dblk maxima)
+    int n_dblk;
+    const uint32_t* x_amax;    // DSC: bits of max |x| per block of the pass that looked for it
     int n_xamax;
     float run_vmax;            // DSC: largest Σ|val| over the entries of one (atom, voxel) run
     const int32_t* chunk_end;  // DSC on the live-entry stream: end of each chunk's entries (else NULL:
@@ -664,44 +653,6 @@ __device__ __forceinline__ void dsc_flush_sq(const TcArgs& A, double& sq, int p,
     sq = 0.0;
 }
 
-// D (Nθ x Na, θ fastest) into shared memory as a BF16 K-major MMA operand,
-// zero-padded to np x kp: ATOM_ROWS (WC: rows = atoms, K = θ) or not (DSC: rows
-// = θ, K = atoms).  Each step moves four θ of one atom with one 16-byte load, and
-// the loop is unrolled so that several loads are in flight.
-template <bool ATOM_ROWS>
-__device__ __forceinline__ void stage_d(const TcArgs& A, unsigned char* dst, uint32_t sbo, int tid, int nthr) {
-    const int q4 = A.np >> 2, n = A.kp * q4;
-    const bool vec = (A.nt & 3) == 0 && (reinterpret_cast<uintptr_t>(A.D) & 15) == 0;
-#pragma unroll 4
-    for (int g = tid; g < n; g += nthr) {
-        const int a = g / q4, t0 = 4 * (g - a * q4);
-        float4 d = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (a < A.na && t0 < A.nt) {
-            const float* src = A.D + (int64_t)A.nt * a + t0;
-            if (vec) {
-                d = __ldg(reinterpret_cast<const float4*>(src));
-            } else {
-                d.x = __ldg(src);
-                if (t0 + 1 < A.nt) d.y = __ldg(src + 1);
-                if (t0 + 2 < A.nt) d.z = __ldg(src + 2);
-                if (t0 + 3 < A.nt) d.w = __ldg(src + 3);
-            }
-        }
-        if (ATOM_ROWS) {
-            const __nv_bfloat162 lo = __floats2bfloat162_rn(d.x, d.y), hi = __floats2bfloat162_rn(d.z, d.w);
-            uint2 v;
-            v.x = *reinterpret_cast<const uint32_t*>(&lo);
-            v.y = *reinterpret_cast<const uint32_t*>(&hi);
-            *reinterpret_cast<uint2*>(dst + kmajor_off(a, t0, sbo)) = v;  // K = θ: 4 consecutive bf16
-        } else {
-            *reinterpret_cast<__nv_bfloat16*>(dst + kmajor_off(t0, a, sbo)) = __float2bfloat16_rn(d.x);
-            *reinterpret_cast<__nv_bfloat16*>(dst + kmajor_off(t0 + 1, a, sbo)) = __float2bfloat16_rn(d.y);
-            *reinterpret_cast<__nv_bfloat16*>(dst + kmajor_off(t0 + 2, a, sbo)) = __float2bfloat16_rn(d.z);
-            *reinterpret_cast<__nv_bfloat16*>(dst + kmajor_off(t0 + 3, a, sbo)) = __float2bfloat16_rn(d.w);
-        }
-    }
-}
-
 // ------------------------------------------------------ FP16 MMA operands
 // The stored precision stays BF16 (Phi values, D); the operands the tensor cores
 // read are FP16 (11 significand bits) under exact power-of-two scales, so that
@@ -719,38 +670,136 @@ __device__ __forceinline__ int f16_scale_exp(uint32_t bound_bits) {
     return max(-120, min(120, 15 - e));
 }
 
-// Bits of max |v| over n BF16 values at p (a multiple of 2).
-__device__ __forceinline__ uint32_t bf16_absmax_bits(const unsigned char* p, uint32_t n, int tid, int nthr) {
-    const uint32_t* q = reinterpret_cast<const uint32_t*>(p);
-    uint32_t m = 0u;
-    for (uint32_t i = tid; i < n / 2; i += nthr) {
-        const uint32_t u = q[i];
-        m = max(m, max((u << 16) & 0x7FFFFFFFu, u & 0x7FFF0000u));
-    }
-    return m;
-}
-
-// n BF16 values at p (a multiple of 2) become FP16 values times 2^k, in place.
-__device__ __forceinline__ void bf16_to_f16_scaled(unsigned char* p, uint32_t n, int k, int tid, int nthr) {
-    uint32_t* q = reinterpret_cast<uint32_t*>(p);
-    const float sc = ldexpf(1.0f, k);
-    for (uint32_t i = tid; i < n / 2; i += nthr) {
-        const uint32_t u = q[i];
-        const __half2 h = __floats2half2_rn(__uint_as_float(u << 16) * sc, __uint_as_float(u & 0xFFFF0000u) * sc);
-        q[i] = *reinterpret_cast<const uint32_t*>(&h);
-    }
-}
-
 __device__ __forceinline__ uint32_t warp_max_u32(uint32_t v) {
     for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
 }
 
-// Bits of max |v| over n floats in global memory.
-__device__ __forceinline__ uint32_t f32_absmax_bits(const float* p, int n, int tid, int nthr) {
+// Largest of n words, by every warp for itself.
+__device__ __forceinline__ uint32_t max_of_parts(const uint32_t* p, int n) {
     uint32_t m = 0u;
-    for (int i = tid; i < n; i += nthr) m = max(m, abs_bits(__ldg(p + i)));
-    return m;
+    for (int i = threadIdx.x & 31; i < n; i += 32) m = max(m, p[i]);
+    return warp_max_u32(m);
+}
+
+// ------------------------------------------------- a call's small preparations
+//
+// One launch before the DSC, or before a WC whose r no DSC of this index wrote,
+// does what every CTA of those kernels would otherwise do for itself:
+//  - D as the MMA operands the CTAs copy into shared memory with one bulk copy each
+//    (BF16 storage: D's BF16 values as FP16 times 2^kD, K-major, once with rows θ for
+//    the DSC and once with rows = atoms for the WC), its scale exponent kD, and per
+//    block of atoms the largest column sum of |D| (WC's fixed-point bound);
+//  - DSC: per block, the bits of max |x| over the finite values of x, the scale of
+//    the FP16 S operand (a NaN or inf weight makes its run sums non-finite whatever
+//    the scale; leaving it out keeps every other S value scaled into FP16's range);
+//  - the zeroes of the g that the next WC adds into.
+// Staged by each CTA from the float32 D (a pass to round and store it, one for its
+// maximum, one to scale it), D took the first 12 us of every DSC launch and 17 us
+// of every WC launch; a copy of the finished operand takes 2 to 3 us, and in the
+// kernels only the thread that issues the MMAs waits for it.
+// Each block of atoms looks for the maximum of all of D itself, so the blocks are
+// large: 1024 threads read the 138 KB of a 96 x 360 D in one round of 16-byte loads
+// (256 threads took the launch 3 us longer).
+constexpr int PREP_THREADS = 1024;
+
+struct PrepArgs {
+    const float* D;
+    unsigned char *img_dsc, *img_wc;  // NULL: FP32 storage (the kernels keep D's parts in tensor memory)
+    uint32_t* info;                   // [0] kD, [1 ..] column-sum maxima per block of atoms
+    const float* x;                   // DSC input, or NULL
+    int64_t n_x;
+    uint32_t* x_amax;
+    float* zero;                      // cleared, or NULL
+    int64_t n_zero;
+    int nt, na, np, kp, n_dblk, n_xblk;
+};
+
+// Part blk of the D work, in blocks of THREADS threads (one atom a warp).
+template <int THREADS>
+__device__ __forceinline__ void prep_d(const PrepArgs& P, int blk) {
+    __shared__ uint32_t dmax_bits, sum_bits;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) dmax_bits = sum_bits = 0u;
+    __syncthreads();
+    uint32_t m = 0u;
+    const int n = P.nt * P.na;
+    if ((reinterpret_cast<uintptr_t>(P.D) & 15) == 0) {
+#pragma unroll 8
+        for (int i = tid; i < n / 4; i += THREADS) m = max(m, absmax4_bits(__ldg(reinterpret_cast<const float4*>(P.D) + i)));
+        for (int i = n / 4 * 4 + tid; i < n; i += THREADS) m = max(m, abs_bits(__ldg(P.D + i)));
+    } else {
+#pragma unroll 8
+        for (int i = tid; i < n; i += THREADS) m = max(m, abs_bits(__ldg(P.D + i)));
+    }
+    m = warp_max_u32(m);
+    if (lane == 0) atomicMax(&dmax_bits, m);
+    __syncthreads();
+    if (!P.img_dsc) {
+        if (blk == 0 && tid == 0) P.info[0] = (uint32_t)f16_scale_exp(dmax_bits);
+        return;
+    }
+    // the largest BF16 |D| is the BF16 rounding of the largest |D|
+    const float dmax = __bfloat162float(__float2bfloat16_rn(__uint_as_float(dmax_bits)));
+    const int kD = f16_scale_exp(abs_bits(dmax));
+    if (blk == 0 && tid == 0) P.info[0] = (uint32_t)kD;
+    const float sc = ldexpf(1.0f, kD);
+    const uint32_t sbo_d = (uint32_t)(P.kp / 8) * 128u, sbo_k = (uint32_t)(P.np / 8) * 128u;
+    const int a = blk * (THREADS / 32) + warp;
+    float sum = 0.0f;
+    for (int t = lane; t < P.np; t += 32) {
+        const float d = a < P.na && t < P.nt ? __bfloat162float(__float2bfloat16_rn(__ldg(P.D + (int64_t)P.nt * a + t))) : 0.0f;
+        const __half h = __float2half_rn(d * sc);
+        *reinterpret_cast<__half*>(P.img_dsc + kmajor_off(t, a, sbo_d)) = h;
+        *reinterpret_cast<__half*>(P.img_wc + kmajor_off(a, t, sbo_k)) = h;
+        sum += fabsf(d);
+    }
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    // (a NaN column sum gives bits above those of +inf)
+    if (lane == 0) atomicMax(&sum_bits, abs_bits(sum));
+    __syncthreads();
+    if (tid == 0) P.info[1 + blk] = sum_bits;
+}
+
+__device__ __forceinline__ void prep_zero(const PrepArgs& P, int64_t i0, int64_t n_thr) {
+    if (!P.zero) return;
+    if ((reinterpret_cast<uintptr_t>(P.zero) & 15) == 0) {
+        for (int64_t i = i0; i < P.n_zero / 4; i += n_thr) reinterpret_cast<float4*>(P.zero)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int64_t i = P.n_zero / 4 * 4 + i0; i < P.n_zero; i += n_thr) P.zero[i] = 0.0f;
+    } else {
+        for (int64_t i = i0; i < P.n_zero; i += n_thr) P.zero[i] = 0.0f;
+    }
+}
+
+// Blocks [0, n_dblk) prepare D, the n_xblk after them x and the zeroes.
+__global__ void __launch_bounds__(PREP_THREADS) tc_prep_kernel(PrepArgs P) {
+    if ((int)blockIdx.x < P.n_dblk) {
+        prep_d<PREP_THREADS>(P, blockIdx.x);
+        return;
+    }
+    const int blk = blockIdx.x - P.n_dblk;
+    const int64_t i0 = blk * (int64_t)PREP_THREADS + threadIdx.x, n_thr = (int64_t)P.n_xblk * PREP_THREADS;
+    prep_zero(P, i0, n_thr);
+    if (!P.x) return;
+    uint32_t m = 0u;
+    auto take = [&](float x) {
+        const uint32_t bits = abs_bits(x);
+        if (bits < 0x7F800000u) m = max(m, bits);
+    };
+    if ((reinterpret_cast<uintptr_t>(P.x) & 15) == 0) {
+#pragma unroll 4
+        for (int64_t i = i0; i < P.n_x / 4; i += n_thr) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(P.x) + i);
+            take(v.x);
+            take(v.y);
+            take(v.z);
+            take(v.w);
+        }
+        for (int64_t i = P.n_x / 4 * 4 + i0; i < P.n_x; i += n_thr) take(__ldg(P.x + i));
+    } else {
+        for (int64_t i = i0; i < P.n_x; i += n_thr) take(__ldg(P.x + i));
+    }
+    block_absmax_out(m, P.x_amax + blk);
 }
 
 // F32 = false: BF16 storage; S (A operand, 128 tile rows x K) and D (B operand)
@@ -767,7 +816,7 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ uint64_t full_bar[DSTAGE], empty_bar[DSTAGE], zero_bar[DSTAGE], acc_full[2], acc_empty[2], fin_bar,
         tab_bar, d_ready;
-    __shared__ uint32_t tmem_base, dmax_bits, xmax_bits;
+    __shared__ uint32_t tmem_base;
     __shared__ int abort_flag, never;
     __shared__ int chunk_next[DSTAGE];  // next dynamically handed-out 256-entry block of the stage's chunk
     __shared__ double red[DSC_EPI_WARPS];
@@ -785,39 +834,7 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
     float* wl = reinterpret_cast<float*>(Ss + DSTAGE * STG);
     float* Ts = wl + ((A.max_fb + 3) / 4 * 4 + 4);  // F32: the epilogue warps' transpose tiles
     const uint32_t SBO_D = (uint32_t)(A.kp / 8) * 128u;
-
-    // BF16 storage: D as the B operand, rows θ (N), K = atoms; BF16 (its stored
-    // precision), zero-padded, then FP16 times 2^kD in place.
-    if (tid == 0) dmax_bits = xmax_bits = 0u;
-    if (!F32) stage_d<false>(A, Ds, SBO_D, tid, blockDim.x);
-    __syncthreads();
-    {
-        // max |D| (for kD) and max |x| over the weight gather's block maxima (for kS)
-        uint32_t dm = F32 ? warp_max_u32(f32_absmax_bits(A.D, A.nt * A.na, tid, blockDim.x))
-                          : warp_max_u32(bf16_absmax_bits(Ds, (uint32_t)A.np * A.kp, tid, blockDim.x));
-        uint32_t xm = 0u;
-        for (int i = tid; i < A.n_xamax; i += blockDim.x) xm = max(xm, A.x_amax[i]);
-        xm = warp_max_u32(xm);
-        if (lane == 0) {
-            atomicMax(&dmax_bits, dm);
-            atomicMax(&xmax_bits, xm);
-        }
-    }
-    __syncthreads();
-    const int kD = f16_scale_exp(dmax_bits);
-    if (!F32) bf16_to_f16_scaled(Ds, (uint32_t)A.np * A.kp, kD, tid, blockDim.x);
-    // S = Σ_run val·x is stored as FP16 times 2^kS, with |S| <= run_vmax · max|x|
-    int kS = 0;
-    {
-        const float xmax = __uint_as_float(xmax_bits);
-        if (xmax_bits != 0u && xmax <= 3.0e38f && A.run_vmax > 0.0f) {
-            int ex = 0, er = 0;
-            (void)frexpf(xmax, &ex);
-            (void)frexpf(A.run_vmax, &er);
-            kS = max(-120, min(120, 15 - ex - er));
-        }
-    }
-    const float s_scale = ldexpf(1.0f, kS), y_unscale = ldexpf(1.0f, -kS - kD);
+    const uint32_t d_copy = (uint32_t)A.np * A.kp * 2;
     if (tid == 0) {
         for (int s = 0; s < DSTAGE; ++s) {
             mbar_init(&full_bar[s], DSC_PROD_WARPS);
@@ -831,11 +848,31 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
             mbar_init(&acc_empty[b], DSC_EPI_WARPS);
         }
         mbar_init(&fin_bar, 1);
-        mbar_init(&d_ready, DSC_MMA_WARP);  // every producer and epilogue warp stores part of D
+        // BF16 storage: one bulk copy; FP32: every producer and epilogue warp stores part of D
+        mbar_init(&d_ready, F32 ? DSC_MMA_WARP : 1);
         abort_flag = 0;
         never = 0;
         fence_barrier_init();
+        if (!F32) {
+            // D as the B operand: rows θ (N), K = atoms, FP16 times 2^kD
+            mbar_arrive_expect_tx(&d_ready, d_copy);
+            bulk_copy_g2s(Ds, A.d_img, d_copy, &d_ready);
+        }
     }
+    const int kD = (int)A.d_info[0];
+    // S = Σ_run val·x is stored as FP16 times 2^kS, with |S| <= run_vmax · max|x|
+    int kS = 0;
+    {
+        const uint32_t xmax_bits = max_of_parts(A.x_amax, A.n_xamax);
+        const float xmax = __uint_as_float(xmax_bits);
+        if (xmax_bits != 0u && xmax <= 3.0e38f && A.run_vmax > 0.0f) {
+            int ex = 0, er = 0;
+            (void)frexpf(xmax, &ex);
+            (void)frexpf(A.run_vmax, &er);
+            kS = max(-120, min(120, 15 - ex - er));
+        }
+    }
+    const float s_scale = ldexpf(1.0f, kS), y_unscale = ldexpf(1.0f, -kS - kD);
     const uint32_t tmem_cols = dsc_tmem_cols(A.kp, F32);
     if (warp == DSC_MMA_WARP) {
         tmem_alloc(&tmem_base, tmem_cols);
@@ -1261,6 +1298,10 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
             mbar_arrive_expect_tx(&zero_bar[z], DS_BYTES);
             bulk_copy_g2s(Ss + z * DS_BYTES, g_zero_chunk, DS_BYTES, &zero_bar[z]);
         }
+        if (!mbar_wait(&d_ready, 0, &never, WAIT_LIMIT)) {  // D has arrived (also before the CTA may exit)
+            abort_flag = 1;
+            stop = true;
+        }
         for (int r = 0; !stop; ++r) {
             const int brick = live_brick(A, G, cta, r);
             if (brick < 0) break;
@@ -1391,13 +1432,20 @@ __device__ __forceinline__ int wseg(const TcArgs& A, int t, int q, int s) {
 // memory so that the loads of r are independent of one another.
 constexpr int AMAX_THREADS = 256;
 
-__global__ void __launch_bounds__(AMAX_THREADS) wc_amax_kernel(TcArgs A) {
+// Blocks [0, P.n_dblk) prepare D for the WC, the others take the tiles and clear g.
+__global__ void __launch_bounds__(AMAX_THREADS) wc_amax_kernel(TcArgs A, PrepArgs P) {
     __shared__ int32_t tv[TILE_V];
     __shared__ uint32_t wmax[AMAX_THREADS / 32];
-    if (!A.bg.live && gate_skip(A.gate, A.gate_mode)) return;
     const int tid = threadIdx.x;
+    if ((int)blockIdx.x < P.n_dblk) {
+        prep_d<AMAX_THREADS>(P, blockIdx.x);
+        return;
+    }
+    const int blk = blockIdx.x - P.n_dblk, n_blk = gridDim.x - P.n_dblk;
+    prep_zero(P, blk * (int64_t)AMAX_THREADS + tid, (int64_t)n_blk * AMAX_THREADS);
+    if (!A.bg.live && gate_skip(A.gate, A.gate_mode)) return;
     const int n_tiles = A.brick_tile_ptr[A.n_bricks];
-    for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+    for (int t = blk; t < n_tiles; t += n_blk) {
         if (A.bg.live) {
             int lo = 0, hi = A.n_bricks - 1;  // the brick of tile t: last brick starting at or before t
             while (lo < hi) {
@@ -1504,8 +1552,8 @@ __device__ __forceinline__ void load_r_tile(const TcArgs& A, int t, const RUnits
 
 __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
     extern __shared__ unsigned char smem_raw[];
-    __shared__ uint64_t r_full[2], r_empty[2], z_full[ZSLOTS], z_empty[ZSLOTS], fin_bar;
-    __shared__ uint32_t tmem_base, d1_bits, dmax_bits;
+    __shared__ uint64_t r_full[2], r_empty[2], z_full[ZSLOTS], z_empty[ZSLOTS], fin_bar, d_ready;
+    __shared__ uint32_t tmem_base;
     __shared__ int abort_flag, never;
     if (!A.bg.live && gate_skip(A.gate, A.gate_mode)) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -1520,8 +1568,6 @@ __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
     float* gl = Zc + 4 * wg * (ZW_BYTES / 4);
     const uint32_t SBO_K = (uint32_t)(A.np / 8) * 128u;  // 8-row groups of both operands (K = θ)
 
-    // D as the B operand: rows = atoms (N), K = θ; bf16, zero-padded.
-    stage_d<true>(A, Dw, SBO_K, tid, blockDim.x);
     if (tid == 0) {
         for (int b = 0; b < 2; ++b) {
             mbar_init(&r_full[b], WC_LOAD_WARPS);
@@ -1532,11 +1578,14 @@ __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
             mbar_init(&z_empty[z], WC_SCAT_WARPS);
         }
         mbar_init(&fin_bar, 1);
+        mbar_init(&d_ready, 1);
         abort_flag = 0;
         never = 0;
-        d1_bits = 0u;
-        dmax_bits = 0u;
         fence_barrier_init();
+        // D as the B operand: rows = atoms (N), K = θ, FP16 times 2^kD
+        const uint32_t d_copy = (uint32_t)A.kp * A.np * 2;
+        mbar_arrive_expect_tx(&d_ready, d_copy);
+        bulk_copy_g2s(Dw, A.d_img, d_copy, &d_ready);
     }
     if (warp == WC_MMA_WARP) {
         tmem_alloc(&tmem_base, 512);
@@ -1548,28 +1597,9 @@ __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
     tc_fence_after();
     const uint32_t tb = tmem_base;
     const int G = gridDim.x, cta = blockIdx.x;
-    {
-        // max over atoms of Σθ |D[θ, a]| for the BF16 D the MMA reads (one warp per
-        // atom; a NaN column sum gives bits above those of +inf)
-        uint32_t m = 0u;
-        for (int a = warp; a < A.na; a += WC_THREADS / 32) {
-            float sum = 0.0f;
-            for (int t = lane; t < A.np; t += 32)
-                sum += fabsf(__bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(Dw + kmajor_off(a, t, SBO_K))));
-            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-            m = max(m, __float_as_uint(sum) & 0x7FFFFFFFu);
-        }
-        if (lane == 0 && m != 0u) atomicMax(&d1_bits, m);
-        const uint32_t dm = warp_max_u32(bf16_absmax_bits(Dw, (uint32_t)A.kp * A.np, tid, blockDim.x));
-        if (lane == 0) atomicMax(&dmax_bits, dm);
-    }
-    __syncthreads();
     // the MMA reads D as FP16 times 2^kD (the BF16 values, exactly); each tile's R
     // as FP16 times 2^kR of its brick, so that Z in tensor memory is 2^(kR+kD) Z
-    const int kD = f16_scale_exp(dmax_bits);
-    bf16_to_f16_scaled(Dw, (uint32_t)A.kp * A.np, kD, tid, blockDim.x);
-    fence_proxy_async_smem();
-    __syncthreads();
+    const int kD = (int)A.d_info[0];
 
     if (warp < WC_SCAT_WARPS) {
         const int q = warp & 3, h = warp >> 2;
@@ -1579,6 +1609,8 @@ __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
         const int kc = A.kp / 128;  // 128-atom chunks per tile
         uint32_t kcount = 0;        // chunks handed over so far (ring position)
         bool dead = false;
+        // max over atoms of Σθ |D[θ, a]| of the BF16 D (NaN above +inf)
+        const float d1 = __uint_as_float(max_of_parts(A.d_info + 1, A.n_dblk));
         for (int r = 0;; ++r) {
             const int brick = live_brick(A, G, cta, r);
             if (brick < 0) break;
@@ -1592,7 +1624,7 @@ __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
             for (int i = 4 * A.brick_tile_ptr[brick] + lane; i < 4 * A.brick_tile_ptr[brick + 1]; i += 32)
                 am = max(am, A.tile_amax[i]);
             for (int o = 16; o > 0; o >>= 1) am = max(am, __shfl_xor_sync(0xffffffffu, am, o));
-            const float bnd = A.brick_cv[brick] * __uint_as_float(d1_bits) * __uint_as_float(am);
+            const float bnd = A.brick_cv[brick] * d1 * __uint_as_float(am);
             int bexp = 0;
             (void)frexpf(bnd, &bexp);
             // (Z·sc < 2^29 / cv must also stay finite: cv >= 1e-28)
@@ -1776,6 +1808,10 @@ __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
         const int kc = A.kp / 128;
         uint32_t tcount = 0, kcount = 0;
         bool stop = false;
+        if (!mbar_wait(&d_ready, 0, &never, WAIT_LIMIT)) {  // D has arrived (also before the CTA may exit)
+            abort_flag = 1;
+            stop = true;
+        }
         for (int r = 0; !stop; ++r) {
             const int brick = live_brick(A, G, cta, r);
             if (brick < 0) break;
@@ -1879,7 +1915,7 @@ __device__ __forceinline__ void wc32_segment(const TcArgs& A, int beg, int end, 
 __global__ void __maxnreg__(96) wc_tc32_kernel(TcArgs A) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ uint64_t r_full[2], r_empty[2], z_full[Z32_SLOTS], z_empty[Z32_SLOTS], fin_bar, d_ready;
-    __shared__ uint32_t tmem_base, dmax_bits;
+    __shared__ uint32_t tmem_base;
     __shared__ int abort_flag, never;
     if (!A.bg.live && gate_skip(A.gate, A.gate_mode)) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -1905,7 +1941,6 @@ __global__ void __maxnreg__(96) wc_tc32_kernel(TcArgs A) {
         mbar_init(&d_ready, 4 * kc);  // the warps that store D's blocks
         abort_flag = 0;
         never = 0;
-        dmax_bits = 0u;
         fence_barrier_init();
     }
     if (warp == WC_MMA_WARP) {
@@ -1918,12 +1953,7 @@ __global__ void __maxnreg__(96) wc_tc32_kernel(TcArgs A) {
     tc_fence_after();
     const uint32_t tb = tmem_base;
     const int G = gridDim.x, cta = blockIdx.x;
-    {
-        const uint32_t dm = warp_max_u32(f32_absmax_bits(A.D, A.nt * A.na, tid, blockDim.x));
-        if (lane == 0) atomicMax(&dmax_bits, dm);
-    }
-    __syncthreads();
-    const int kD = f16_scale_exp(dmax_bits);
+    const int kD = (int)A.d_info[0];
 
     if (warp < WC_SCAT_WARPS) {
         const int q = warp & 3, h = warp >> 2;  // atoms 32q .. of each block; row quarters h, h + wg, ...
@@ -2200,8 +2230,30 @@ static TcArgs make_args(life_index_s* ix) {
     return A;
 }
 
+// What the kernels of one call read besides the layout: D's operands and scale, and
+// (for a DSC) max |x|; zero (nf floats, or NULL) is cleared on the way.
+static PrepArgs prep_args(life_index_s* ix, const float* D, float* zero, int threads) {
+    TileLayout& L = ix->tile;
+    PrepArgs P{};
+    P.D = D;
+    if (L.vbytes == 2) {
+        P.img_dsc = L.d_img.as<unsigned char>();
+        P.img_wc = P.img_dsc + (size_t)L.np * L.kp * 2;
+    }
+    P.info = L.d_info.as<uint32_t>();
+    P.zero = zero;
+    P.n_zero = zero ? ix->nf : 0;
+    P.nt = ix->nt;
+    P.na = ix->na;
+    P.np = L.np;
+    P.kp = L.kp;
+    P.n_dblk = L.vbytes == 2 ? L.kp / (threads / 32) : 1;
+    return P;
+}
+
 life_status dsc_tc(life_index_s* ix, const float* D, const float* w, const float* b, float* y, double* partial,
-                   int* n_partial, const life_sbb_state* gate, int gate_mode, cudaStream_t s, const BatchGate& bg) {
+                   int* n_partial, const life_sbb_state* gate, int gate_mode, cudaStream_t s, const BatchGate& bg,
+                   float* zero) {
     TcArgs A = make_args(ix);
     A.bg = bg;
     if (!A.status) {
@@ -2224,26 +2276,34 @@ life_status dsc_tc(life_index_s* ix, const float* D, const float* w, const float
     }
     const uint32_t smem = dsc_smem_bytes(A.np, A.kp, A.max_fb, f32);
     const bool sparse = L.sparse && !bg.live && L.wb_total > 0 && L.n_nnz > 0;
-    if (L.wb_total > 0) {
-        if (sparse)
-            // the last block decides: full or compacted stream, rebuild or not (the
-            // SBB step's DSC of w never rebuilds: its support lies inside that of the
-            // previous projected gradient; the DSC of the projected gradient rebuilds
-            // with the backoff; a public call whenever its input needs it)
-            wb_gather_live_kernel<<<ix->num_sms * 8, GATHER_THREADS, 0, s>>>(
-                L.wb_src.as<int32_t>(), L.wb_total, w, L.wb.as<float>(), L.wb_live.as<uint8_t>(),
-                L.sparse_ctl.as<SparseCtl>(), (unsigned long long)L.n_brick_slots,
-                !gate ? ALLOW_FREE : (gate_mode == GATE_ACTIVE ? ALLOW_NONE : ALLOW_BACKOFF), gate, gate_mode,
-                L.x_amax.as<uint32_t>());
-        else
-            // the DSC gathers each brick's weights itself; this pass only finds max |w|
-            x_amax_kernel<<<ix->num_sms, 256, 0, s>>>(w, ix->nf, L.x_amax.as<uint32_t>());
-        A.x_amax = L.x_amax.as<uint32_t>();
-        A.n_xamax = sparse ? ix->num_sms * 8 : ix->num_sms;
-        A.gather_w = sparse ? 0 : 1;
-        A.wb_src = L.wb_src.as<int32_t>();
+    if (sparse) {
+        // the last block decides: full or compacted stream, rebuild or not (the
+        // SBB step's DSC of w never rebuilds: its support lies inside that of the
+        // previous projected gradient; the DSC of the projected gradient rebuilds
+        // with the backoff; a public call whenever its input needs it)
+        wb_gather_live_kernel<<<ix->num_sms * 8, GATHER_THREADS, 0, s>>>(
+            L.wb_src.as<int32_t>(), L.wb_total, w, L.wb.as<float>(), L.wb_live.as<uint8_t>(),
+            L.sparse_ctl.as<SparseCtl>(), (unsigned long long)L.n_brick_slots,
+            !gate ? ALLOW_FREE : (gate_mode == GATE_ACTIVE ? ALLOW_NONE : ALLOW_BACKOFF), gate, gate_mode,
+            L.x_amax.as<uint32_t>());
         LIFE_CHECK_LAUNCH();
     }
+    PrepArgs P = prep_args(ix, D, zero, PREP_THREADS);
+    if (!sparse) {  // the DSC gathers each brick's weights itself: this pass finds max |w|
+        P.x = w;
+        P.n_x = ix->nf;
+        P.x_amax = L.x_amax.as<uint32_t>();
+    }
+    P.n_xblk = ix->num_sms;
+    tc_prep_kernel<<<P.n_dblk + P.n_xblk, PREP_THREADS, 0, s>>>(P);
+    LIFE_CHECK_LAUNCH();
+    A.x_amax = L.x_amax.as<uint32_t>();
+    A.n_xamax = sparse ? ix->num_sms * 8 : P.n_xblk;
+    A.gather_w = sparse ? 0 : 1;
+    A.wb_src = L.wb_src.as<int32_t>();
+    A.d_img = P.img_dsc;
+    A.d_info = P.info;
+    A.n_dblk = P.n_dblk;
     auto kern = f32 ? dsc_tc_kernel<true> : dsc_tc_kernel<false>;
     LIFE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int grid = (int)std::min<int64_t>(ix->num_sms, L.n_bricks);
@@ -2320,8 +2380,16 @@ life_status wc_tc(life_index_s* ix, const float* D, const float* r, float* g, co
     const uint32_t smem = wc_smem_bytes(A.np, A.kp, A.max_fb, A.wgroups, A.rbufs, f32);
     auto kern = f32 ? wc_tc32_kernel : wc_tc_kernel;
     LIFE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (ix->tile.n_tiles > 0 && !r_is_dsc_out) {
-        wc_amax_kernel<<<(unsigned)std::min<int64_t>(ix->tile.n_tiles, (int64_t)ix->num_sms * 8), AMAX_THREADS, 0, s>>>(A);
+    // (blocks as in the launch that wrote d_info: the DSC's, or this call's own)
+    const PrepArgs P = prep_args(ix, D, g, r_is_dsc_out ? PREP_THREADS : AMAX_THREADS);
+    A.d_img = P.img_wc;
+    A.d_info = P.info;
+    A.n_dblk = P.n_dblk;
+    if (!r_is_dsc_out) {
+        // (after a DSC of this index that wrote r, its epilogue left the tiles' maxima and
+        // its preparations D's operands and the zeroed g)
+        const int64_t blk = std::min<int64_t>(std::max<int64_t>(ix->tile.n_tiles, 1), (int64_t)ix->num_sms * 8);
+        wc_amax_kernel<<<(unsigned)(P.n_dblk + blk), AMAX_THREADS, 0, s>>>(A, P);
         LIFE_CHECK_LAUNCH();
     }
     const int grid = (int)std::min<int64_t>(ix->num_sms, ix->tile.n_bricks);

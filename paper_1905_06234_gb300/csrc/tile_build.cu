@@ -932,6 +932,8 @@ life_status build_tile_layout(life_index_s* ix, cudaStream_t s) {
     }
     LIFE_TRY(L.x_amax.alloc(sizeof(uint32_t) * (size_t)std::max(ix->num_sms, 1) * 8));
     LIFE_CUDA_TRY(cudaMemsetAsync(L.x_amax.p, 0, sizeof(uint32_t) * (size_t)std::max(ix->num_sms, 1) * 8, s));
+    if (L.vbytes == 2) LIFE_TRY(L.d_img.alloc((size_t)2 * L.np * L.kp * 2));
+    LIFE_TRY(L.d_info.alloc(sizeof(uint32_t) * (size_t)(1 + L.kp / 8)));
     // live-entry DSC stream: allocated at full size, filled on demand by a DSC call
     L.sparse = ix->sparse_dsc != 0 && !grouped;
     if (L.sparse) {
