@@ -241,9 +241,9 @@ LIFE_API life_status life_dsc_grad_D(life_index idx, const float* gy, const floa
  * The same dL/dD as life_dsc_grad_D, for callers that may not allocate device
  * memory while they run: code being captured into a CUDA graph, where cudaMalloc
  * is not allowed, or a real-time loop that allocates only at start-up.
- * life_dsc_grad_D allocates temporary memory on every call for its split-K
- * partial sums; this entry point allocates nothing and keeps those sums in a
- * fixed device array compiled into the library instead.  The paper has no
+ * life_dsc_grad_D keeps its split-K partial sums in memory of the index, which its
+ * first call allocates; this entry point allocates nothing on any call and keeps
+ * those sums in a fixed device array compiled into the library instead.  The paper has no
  * counterpart to this call.
  *  - Limit: (number of atom chunks) x Nθ <= 2^20 floats (the array is 4 MiB, held
  *    on every GPU that loads the library until the process exits); a larger index

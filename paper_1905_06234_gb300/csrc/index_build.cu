@@ -651,6 +651,7 @@ life_status build_atom_layout(life_index_s* ix, cudaStream_t s) {
     LIFE_TRY(A.chunk_beg.alloc(sizeof(int32_t) * cbeg.size()));
     LIFE_TRY(A.chunk_atom.alloc(sizeof(int32_t) * (catom.size() + 1)));
     LIFE_TRY(A.atom_chunk.alloc(sizeof(int32_t) * achunk.size()));
+    LIFE_TRY(A.partial.alloc(sizeof(float) * catom.size() * (size_t)ix->nt));
     LIFE_CUDA_TRY(cudaMemcpyAsync(A.chunk_beg.p, cbeg.data(), sizeof(int32_t) * cbeg.size(), cudaMemcpyHostToDevice, s));
     if (!catom.empty())
         LIFE_CUDA_TRY(cudaMemcpyAsync(A.chunk_atom.p, catom.data(), sizeof(int32_t) * catom.size(),

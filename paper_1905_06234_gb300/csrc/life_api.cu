@@ -233,7 +233,7 @@ extern "C" life_status life_index_get_info(life_index idx, life_index_info* out)
     I.n_bricks = idx->tile.n_bricks;
     const DevBuf* bufs[] = {&idx->uval, &idx->voxel_ijk, &idx->vox.vox_ptr, &idx->vox.atom,
                             &idx->vox.fasc, &idx->vox.val, &idx->atoml.voxel, &idx->atoml.fasc, &idx->atoml.val,
-                            &idx->atoml.chunk_beg, &idx->atoml.chunk_atom, &idx->atoml.atom_chunk,
+                            &idx->atoml.chunk_beg, &idx->atoml.chunk_atom, &idx->atoml.atom_chunk, &idx->atoml.partial,
                             &idx->tile.tile_vox, &idx->tile.chunk_ptr, &idx->tile.brick_tile_ptr,
                             &idx->tile.brick_fasc_ptr, &idx->tile.brick_fasc, &idx->tile.brick_order,
                             &idx->tile.soff, &idx->tile.fl, &idx->tile.val, &idx->tile.wkey,

@@ -130,6 +130,7 @@ struct AtomLayout {
     DevBuf chunk_beg;   // int32 [n_chunks+1] nonzero offsets; every chunk lies in one atom
     DevBuf chunk_atom;  // int32 [n_chunks]
     DevBuf atom_chunk;  // int32 [Na+1] chunk offsets per atom
+    DevBuf partial;     // float [n_chunks * Nθ] partial sums of life_dsc_grad_D
     int32_t n_chunks = 0;
 };
 

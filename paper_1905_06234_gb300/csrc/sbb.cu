@@ -73,8 +73,21 @@ life_status sumsq_f32(const float* x, int64_t n, double* partial, int* n_partial
 
 __global__ void dot_f32_kernel(const float* __restrict__ x, const float* __restrict__ y, int64_t n,
                                double* __restrict__ out) {
+    // one block, so the order of the sum is fixed; 8 pairs a thread in flight (one at a
+    // time, the 34560 pairs of a 96 x 360 D took 34 us)
     double s = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) s += (double)x[i] * (double)y[i];
+    int64_t i = threadIdx.x;
+    for (; i + 7 * (int64_t)blockDim.x < n; i += 8 * (int64_t)blockDim.x) {
+        float a[8], b[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            a[e] = __ldg(x + i + e * (int64_t)blockDim.x);
+            b[e] = __ldg(y + i + e * (int64_t)blockDim.x);
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) s += (double)a[e] * (double)b[e];
+    }
+    for (; i < n; i += blockDim.x) s += (double)x[i] * (double)y[i];
     const double t = block_reduce(s);
     if (threadIdx.x == 0) *out = t;
 }
