@@ -1396,16 +1396,21 @@ __host__ __device__ inline uint32_t wc_smem_bytes(int np, int kp, int max_fb, in
 template <bool CHECK, bool FIXED>
 __device__ __forceinline__ void wc_slot_t(const EntrySlot& s, int base, int beg, int end, const float* Zw,
                                           float* gl, uint32_t gl_s) {
+    // all reads of Z before the first add: a read is not moved up past an add to the
+    // table (they could overlap for all the compiler knows), and one after the other
+    // they are a chain of eight round trips to shared memory
+    float x[SLOT];
+#pragma unroll
+    for (int e = 0; e < SLOT; ++e)
+        x[e] = bf16_at(s.val, e) * *reinterpret_cast<const float*>(reinterpret_cast<const char*>(Zw) + u16_at(s.key, e));
 #pragma unroll
     for (int e = 0; e < SLOT; ++e) {
         if (CHECK) {
             const int idx = base + e;
             if (idx < beg || idx >= end) continue;
         }
-        const float z = *reinterpret_cast<const float*>(reinterpret_cast<const char*>(Zw) + u16_at(s.key, e));
-        const float x = bf16_at(s.val, e) * z;
-        if (FIXED) atomicAdd(reinterpret_cast<int*>(reinterpret_cast<char*>(gl) + u16_at(s.fl, e)), __float2int_rn(x));
-        else red_add_shared_f32(gl_s + u16_at(s.fl, e), x);
+        if (FIXED) atomicAdd(reinterpret_cast<int*>(reinterpret_cast<char*>(gl) + u16_at(s.fl, e)), __float2int_rn(x[e]));
+        else red_add_shared_f32(gl_s + u16_at(s.fl, e), x[e]);
     }
 }
 
@@ -1871,15 +1876,19 @@ constexpr int Z32_SLOTS = 3;
 template <bool CHECK>
 __device__ __forceinline__ void wc32_slot_t(const EntrySlot32& s, int base, int beg, int end, const float* Zw,
                                             uint32_t gl_s) {
+    // (reads before adds, as in wc_slot_t)
+    float x[SLOT];
+#pragma unroll
+    for (int e = 0; e < SLOT; ++e)
+        // key: byte offset of (atom, row) in the atom-major Z tile, which holds Z·sc
+        x[e] = slot_val(s, e) * *reinterpret_cast<const float*>(reinterpret_cast<const char*>(Zw) + u16_at(s.key, e));
 #pragma unroll
     for (int e = 0; e < SLOT; ++e) {
         if (CHECK) {
             const int idx = base + e;
             if (idx < beg || idx >= end) continue;
         }
-        // key: byte offset of (atom, row) in the atom-major Z tile, which holds Z·sc
-        const float z = *reinterpret_cast<const float*>(reinterpret_cast<const char*>(Zw) + u16_at(s.key, e));
-        red_add_shared_f32(gl_s + u16_at(s.fl, e), slot_val(s, e) * z);
+        red_add_shared_f32(gl_s + u16_at(s.fl, e), x[e]);
     }
 }
 
