@@ -80,7 +80,7 @@ life_status batch_finalize(life_index_s* ix, cudaStream_t s) {
     const int n = bi.n;
     bi.part_off.assign(n + 1, 0);
     if (ix->algo == LIFE_ALGO_TC && ix->tile.built) {
-        bi.tc_grid = (int32_t)std::max<int64_t>(1, std::min<int64_t>(ix->num_sms, ix->tile.n_bricks));
+        bi.tc_grid = ix->tile.grid;
         bi.simt_grid = 0;
         const int epi = 4;  // epilogue warps of the DSC kernel
         for (int p = 0; p <= n; ++p) bi.part_off[p] = p * bi.tc_grid * epi;

@@ -154,6 +154,9 @@ struct TileLayout {
     DevBuf brick_fasc_ptr;   // int32 [n_bricks + 1] offsets into brick_fasc
     DevBuf brick_fasc;       // int32 [sum] global fascicle id of each brick-local fascicle
     DevBuf brick_order;      // int32 [n_bricks] bricks by decreasing entry count
+    int32_t grid = 0;        // CTAs of an SpMV launch
+    int32_t n_units = 0;
+    DevBuf units;            // int32 [grid + 1] units of each CTA, then per unit its brick, first tile, end tile
     DevBuf soff;             // uint16 [n_nnz]: byte offset of (row, atom mod 128) in a DSC S chunk | 0x8000
                              // if the entry has the same (atom, row) as the previous one
     // WC streams, ordered (tile, row quarter, atom, row, fascicle)

@@ -4,7 +4,8 @@
 // dictionary (Eq. 3: M_v = D Phi_v):
 //   DSC  y[:,v] = D · S[:,v],   S[a,v] = Σ_f val·w[f]        (S built in shared memory)
 //   WC   Z[a,v] = (Dᵀ r[:,v])[a],  g[f] += val·Z[a,v]         (Z read back from TMEM)
-// One CTA per SM walks spatial bricks of voxels (largest first, snake order).
+// One CTA per SM walks work units: spatial bricks of voxels, or runs of a brick's
+// tiles where there are too few bricks to share out evenly.
 // A brick's fascicles are renumbered locally so that w is gathered, and g is
 // accumulated, in shared memory: each global gather or atomic then serves all of
 // a fascicle's entries inside the brick instead of one entry.
@@ -351,7 +352,8 @@ struct TcArgs {
     const int32_t* brick_tile_ptr;
     const int32_t* brick_fasc_ptr;
     const int32_t* brick_fasc;
-    const int32_t* brick_order;
+    const int32_t* cta_unit;   // [grid + 1] work units of each CTA
+    const int32_t *u_brick, *u_t0, *u_t1;  // per unit: its brick and its tiles [t0, t1) of it
     const uint16_t* soff;
     const uint16_t* fl;
     const __nv_bfloat16* val;
@@ -393,21 +395,14 @@ struct TcArgs {
                          // partial sums go to partial[(p * grid + cta) * DSC_EPI_WARPS + epilogue warp]
 };
 
-// Brick processed by CTA c in round r (snake over the size-sorted list), or -1.
-__device__ __forceinline__ int brick_at(int r, int G, int c, int nb) {
-    const int k = r * G + ((r & 1) ? (G - 1 - c) : c);
-    return k < nb ? k : -1;
-}
-
-// The first brick of this CTA at round >= r whose problem is live (r is advanced
+// The first work unit of this CTA at round >= r whose problem is live (r is advanced
 // to its round); -1 when none is left.  Every role of a CTA walks the same
 // sequence, since the problem states do not change during a launch.
-__device__ __forceinline__ int live_brick(const TcArgs& A, int G, int cta, int& r) {
+__device__ __forceinline__ int live_unit(const TcArgs& A, int cta, int& r) {
     for (;; ++r) {
-        const int k = brick_at(r, G, cta, A.n_bricks);
-        if (k < 0) return -1;
-        const int brick = A.brick_order[k];
-        if (!A.bg.live || batch_live(A.bg, A.bg.brick_prob[brick], A.gate_mode)) return brick;
+        const int u = A.cta_unit[cta] + r;
+        if (u >= A.cta_unit[cta + 1]) return -1;
+        if (!A.bg.live || batch_live(A.bg, A.bg.brick_prob[A.u_brick[u]], A.gate_mode)) return u;
     }
 }
 
@@ -484,19 +479,19 @@ __device__ __forceinline__ int chunk_end(const TcArgs& A, int t, int c, int n_c)
     return A.chunk_end ? A.chunk_end[(int64_t)t * n_c + c] : A.chunk_ptr[(int64_t)t * n_c + c + 1];
 }
 
-// Advances (r, brick, t, c) to the CTA's next chunk; false when none is left.
-__device__ __forceinline__ bool next_chunk(const TcArgs& A, int G, int cta, int n_c, int& r, int& brick, int& t,
-                                           int& c, bool& new_brick) {
-    new_brick = false;
+// Advances (r, unit, t, c) to the CTA's next chunk; false when none is left.
+__device__ __forceinline__ bool next_chunk(const TcArgs& A, int cta, int n_c, int& r, int& unit, int& t, int& c,
+                                           bool& new_unit) {
+    new_unit = false;
     if (++c < n_c) return true;
     c = 0;
-    if (++t < A.brick_tile_ptr[brick + 1]) return true;
+    if (++t < A.u_t1[unit]) return true;
     ++r;
-    const int nb = live_brick(A, G, cta, r);
-    if (nb < 0) return false;
-    brick = nb;
-    t = A.brick_tile_ptr[brick];
-    new_brick = true;
+    const int nu = live_unit(A, cta, r);
+    if (nu < 0) return false;
+    unit = nu;
+    t = A.u_t0[unit];
+    new_unit = true;
     return true;
 }
 
@@ -917,9 +912,9 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
     if (warp < DSC_PROD_WARPS) {
         // ---------------- producers: S[a, row] = Σ val·w for one 128-atom chunk
         int r = 0;
-        const int b0 = live_brick(A, G, cta, r);
-        if (b0 >= 0) {
-            int brick = b0, t = A.brick_tile_ptr[brick], c = 0;
+        const int u0 = live_unit(A, cta, r);
+        if (u0 >= 0) {
+            int unit = u0, t = A.u_t0[unit], c = 0;
             int beg = chunk_beg(A, t, 0, n_c), end = chunk_end(A, t, 0, n_c);
             int base = (beg & ~7) + tid * SLOT;
             bool have = base < end;
@@ -939,7 +934,7 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
                         // the brick's weights straight from x: slot i holds x[wb_src[o + i]]
                         // (0 for padding); GW slots a round, loads first
                         constexpr int GW = 8;
-                        const int o = A.wb_ptr[brick], nb4 = A.wb_ptr[brick + 1] - o;
+                        const int o = A.wb_ptr[A.u_brick[unit]], nb4 = A.wb_ptr[A.u_brick[unit] + 1] - o;
                         for (int i0 = tid; i0 < nb4; i0 += GW * DSC_PROD_THREADS) {
                             int32_t id[GW];
 #pragma unroll
@@ -956,15 +951,15 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
                         }
                         // the next brick's slot indices into L2 (they come from DRAM)
                         int rn = r + 1;
-                        const int nbk = live_brick(A, G, cta, rn);
-                        if (nbk >= 0) {
-                            const int o2 = A.wb_ptr[nbk], n2 = A.wb_ptr[nbk + 1] - o2;
+                        const int un = live_unit(A, cta, rn);
+                        if (un >= 0) {
+                            const int o2 = A.wb_ptr[A.u_brick[un]], n2 = A.wb_ptr[A.u_brick[un] + 1] - o2;
                             for (int i = 32 * tid; i < n2; i += 32 * DSC_PROD_THREADS) prefetch_l2(A.wb_src + o2 + i);
                         }
                         named_bar_sync(1, DSC_PROD_THREADS);  // the table is complete
                     } else {
                         if (tid == 0) {  // one bulk copy of the brick's gathered weights
-                            const int o = A.wb_ptr[brick], nb4 = A.wb_ptr[brick + 1] - o;
+                            const int o = A.wb_ptr[A.u_brick[unit]], nb4 = A.wb_ptr[A.u_brick[unit] + 1] - o;
                             mbar_arrive_expect_tx(&tab_bar, 4u * (uint32_t)nb4);
                             if (nb4 > 0) bulk_copy_g2s(wl, A.wb + o, 4u * (uint32_t)nb4, &tab_bar);
                         }
@@ -983,9 +978,9 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
                     abort_flag = 1;
                     dead = true;
                 }
-                int nr = r, nbrick = brick, nt = t, nc = c;
+                int nr = r, nunit = unit, nt = t, nc = c;
                 bool nnew = false;
-                const bool nvalid = next_chunk(A, G, cta, n_c, nr, nbrick, nt, nc, nnew);
+                const bool nvalid = next_chunk(A, cta, n_c, nr, nunit, nt, nc, nnew);
                 int nbeg = 0, nend = 0;
                 if (nvalid) {
                     nbeg = chunk_beg(A, nt, nc, n_c);
@@ -1027,7 +1022,7 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
                 ++cc;
                 if (!nvalid) break;
                 r = nr;
-                brick = nbrick;
+                unit = nunit;
                 t = nt;
                 c = nc;
                 beg = nbeg;
@@ -1051,18 +1046,18 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
         if (A.bg.live && lane == 0 && A.partial)
             for (int p = 0; p < A.bg.n; ++p) A.partial[((int64_t)p * G + cta) * DSC_EPI_WARPS + q] = 0.0;
         for (int r = 0; !stop; ++r) {
-            const int brick = live_brick(A, G, cta, r);
-            if (brick < 0) break;
+            const int unit = live_unit(A, cta, r);
+            if (unit < 0) break;
             bool wy = write_y;
             if (A.bg.live) {
-                const int p = A.bg.brick_prob[brick];
+                const int p = A.bg.brick_prob[A.u_brick[unit]];
                 wy = write_y && batch_writes_y(A.bg, p, A.gate_mode);
                 if (p != cur_p) {
                     if (cur_p >= 0) dsc_flush_sq(A, sq, cur_p, G, cta, q, lane);
                     cur_p = p;
                 }
             }
-            for (int t = A.brick_tile_ptr[brick]; t < A.brick_tile_ptr[brick + 1]; ++t) {
+            for (int t = A.u_t0[unit]; t < A.u_t1[unit]; ++t) {
                 const uint32_t ab = tcount % NACC, aph = (tcount / NACC) & 1u;
                 int vj[4];  // F32: voxel of tile row 32·g + lane
                 if constexpr (F32) {
@@ -1245,9 +1240,9 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
         }
         tc_fence_after();
         for (int r = 0; !stop; ++r) {
-            const int brick = live_brick(A, G, cta, r);
-            if (brick < 0) break;
-            for (int t = A.brick_tile_ptr[brick]; t < A.brick_tile_ptr[brick + 1] && !stop; ++t) {
+            const int unit = live_unit(A, cta, r);
+            if (unit < 0) break;
+            for (int t = A.u_t0[unit]; t < A.u_t1[unit] && !stop; ++t) {
                 if (!mbar_wait(&acc_empty[0], (tcount & 1u) ^ 1u, &abort_flag, WAIT_LIMIT)) {
                     abort_flag = 1;
                     stop = true;
@@ -1303,9 +1298,9 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
             stop = true;
         }
         for (int r = 0; !stop; ++r) {
-            const int brick = live_brick(A, G, cta, r);
-            if (brick < 0) break;
-            for (int t = A.brick_tile_ptr[brick]; t < A.brick_tile_ptr[brick + 1] && !stop; ++t) {
+            const int unit = live_unit(A, cta, r);
+            if (unit < 0) break;
+            for (int t = A.u_t0[unit]; t < A.u_t1[unit] && !stop; ++t) {
                 const uint32_t ab = tcount & 1u, aph = (tcount >> 1) & 1u;
                 if (!mbar_wait(&acc_empty[ab], aph ^ 1u, &abort_flag, WAIT_LIMIT)) { abort_flag = 1; stop = true; break; }
                 tc_fence_after();
@@ -1617,8 +1612,9 @@ __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
         // max over atoms of Σθ |D[θ, a]| of the BF16 D (NaN above +inf)
         const float d1 = __uint_as_float(max_of_parts(A.d_info + 1, A.n_dblk));
         for (int r = 0;; ++r) {
-            const int brick = live_brick(A, G, cta, r);
-            if (brick < 0) break;
+            const int unit = live_unit(A, cta, r);
+            if (unit < 0) break;
+            const int brick = A.u_brick[unit];
             const int fb0 = A.brick_fasc_ptr[brick], nfb = A.brick_fasc_ptr[brick + 1] - fb0;
             // Fixed point: every entry adds val·Z with |val·Z| <= max|val|·max_a Σθ|D|·max|r|
             // (up to the BF16 roundings of r and D, < 1 %), and a fascicle has at most
@@ -1626,7 +1622,7 @@ __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
             // sc = 2^(29 - e), bnd < 2^e, a table word stays below 2^29·1.01 + cnt/2 < 2^31.
             // Non-finite or tiny bounds keep the FP32 table.
             uint32_t am = 0u;
-            for (int i = 4 * A.brick_tile_ptr[brick] + lane; i < 4 * A.brick_tile_ptr[brick + 1]; i += 32)
+            for (int i = 4 * A.u_t0[unit] + lane; i < 4 * A.u_t1[unit]; i += 32)
                 am = max(am, A.tile_amax[i]);
             for (int o = 16; o > 0; o >>= 1) am = max(am, __shfl_xor_sync(0xffffffffu, am, o));
             const float bnd = A.brick_cv[brick] * d1 * __uint_as_float(am);
@@ -1644,7 +1640,7 @@ __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
             if (named_bar_or(2, WC_SCAT_THREADS, dead || abort_flag != 0)) break;
             for (int i = tid; i < nfb; i += WC_SCAT_THREADS) gl[i] = 0.0f;
             named_bar_sync(2, WC_SCAT_THREADS);
-            const int t0 = A.brick_tile_ptr[brick], t1 = A.brick_tile_ptr[brick + 1];
+            const int t0 = A.u_t0[unit], t1 = A.u_t1[unit];
             // this warp's segments in order: (t, s) for t in the brick, s = h, h + wg, ...;
             // a warp step covers two 256-entry blocks (lane i: entries 8i.. of each),
             // and the step after it (or the next segment's first) is loaded while the
@@ -1749,15 +1745,15 @@ __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
         uint32_t tcount = 0;
         bool stop = false;
         for (int r = 0; !stop; ++r) {
-            const int brick = live_brick(A, G, cta, r);
-            if (brick < 0) break;
+            const int unit = live_unit(A, cta, r);
+            if (unit < 0) break;
             int r_next = r + 1;
-            const int next_brick = live_brick(A, G, cta, r_next);
+            const int next_unit = live_unit(A, cta, r_next);
             uint32_t am = 0u;
-            for (int i = 4 * A.brick_tile_ptr[brick] + lane; i < 4 * A.brick_tile_ptr[brick + 1]; i += 32)
+            for (int i = 4 * A.u_t0[unit] + lane; i < 4 * A.u_t1[unit]; i += 32)
                 am = max(am, A.tile_amax[i]);
             const float rs = ldexpf(1.0f, f16_scale_exp(warp_max_u32(am)));
-            for (int t = A.brick_tile_ptr[brick]; t < A.brick_tile_ptr[brick + 1]; ++t) {
+            for (int t = A.u_t0[unit]; t < A.u_t1[unit]; ++t) {
                 // R buffer rb, used for the k-th time (tiles go round the buffers)
                 const uint32_t rb = A.rbufs == 2 ? (tcount & 1u) : 0u, rk = A.rbufs == 2 ? (tcount >> 1) : tcount;
                 unsigned char* Rb = Rs + rb * r_bytes;
@@ -1781,16 +1777,16 @@ __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&r_full[rb]);
                 ++tcount;
-                tv = t + 1 < A.brick_tile_ptr[brick + 1] ? t + 1 : next_brick >= 0 ? A.brick_tile_ptr[next_brick] : t;
+                tv = t + 1 < A.u_t1[unit] ? t + 1 : next_unit >= 0 ? A.u_t0[next_unit] : t;
                 load_r_voxels(A, tv, lt, RU, vv);  // of the tile after this one
                 // pull the voxel rows of r of the tile A.rbufs ahead into L2 (the
                 // loader runs A.rbufs - 1 tiles ahead of the tensor cores), so that
                 // loading it later is not a chain of DRAM round trips
                 int tn = t + A.rbufs;
-                if (tn >= A.brick_tile_ptr[brick + 1]) {
-                    tn -= A.brick_tile_ptr[brick + 1];
-                    tn = (next_brick >= 0 && A.brick_tile_ptr[next_brick] + tn < A.brick_tile_ptr[next_brick + 1])
-                             ? A.brick_tile_ptr[next_brick] + tn : -1;
+                if (tn >= A.u_t1[unit]) {
+                    tn -= A.u_t1[unit];
+                    tn = (next_unit >= 0 && A.u_t0[next_unit] + tn < A.u_t1[next_unit])
+                             ? A.u_t0[next_unit] + tn : -1;
                 }
                 if (tn >= 0) {
                     const int32_t* tvn = A.tile_vox + (int64_t)tn * TILE_V;
@@ -1818,9 +1814,9 @@ __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
             stop = true;
         }
         for (int r = 0; !stop; ++r) {
-            const int brick = live_brick(A, G, cta, r);
-            if (brick < 0) break;
-            for (int t = A.brick_tile_ptr[brick]; t < A.brick_tile_ptr[brick + 1] && !stop; ++t) {
+            const int unit = live_unit(A, cta, r);
+            if (unit < 0) break;
+            for (int t = A.u_t0[unit]; t < A.u_t1[unit] && !stop; ++t) {
                 const uint32_t rb = A.rbufs == 2 ? (tcount & 1u) : 0u, rk = A.rbufs == 2 ? (tcount >> 1) : tcount;
                 const uint32_t sR = sR0 + rb * r_bytes;
                 if (!mbar_wait(&r_full[rb], rk & 1u, &abort_flag, WAIT_LIMIT)) {
@@ -1998,11 +1994,12 @@ __global__ void __maxnreg__(96) wc_tc32_kernel(TcArgs A) {
         uint32_t kcount = 0;  // Z slots handed over so far (ring position)
         bool dead = false;
         for (int r = 0;; ++r) {
-            const int brick = live_brick(A, G, cta, r);
-            if (brick < 0) break;
+            const int unit = live_unit(A, cta, r);
+            if (unit < 0) break;
+            const int brick = A.u_brick[unit];
             const int fb0 = A.brick_fasc_ptr[brick], nfb = A.brick_fasc_ptr[brick + 1] - fb0;
             uint32_t am = 0u;
-            for (int i = 4 * A.brick_tile_ptr[brick] + lane; i < 4 * A.brick_tile_ptr[brick + 1]; i += 32)
+            for (int i = 4 * A.u_t0[unit] + lane; i < 4 * A.u_t1[unit]; i += 32)
                 am = max(am, A.tile_amax[i]);
             am = warp_max_u32(am);
             // Z in tensor memory is 2^(kR + kD)·Z (kR from the brick's max |r|, as the loader scales R)
@@ -2011,7 +2008,7 @@ __global__ void __maxnreg__(96) wc_tc32_kernel(TcArgs A) {
             if (named_bar_or(2, WC_SCAT_THREADS, dead || abort_flag != 0)) break;
             for (int i = tid; i < nfb; i += WC_SCAT_THREADS) gl[i] = 0.0f;
             named_bar_sync(2, WC_SCAT_THREADS);
-            const int t0 = A.brick_tile_ptr[brick], t1 = A.brick_tile_ptr[brick + 1];
+            const int t0 = A.u_t0[unit], t1 = A.u_t1[unit];
             for (int t = t0; t < t1 && !dead; ++t) {
                 // segment bounds of the tile: lane i holds wseg(t, rq, i) for this warp's k-th row quarter rq
                 int bq[4];
@@ -2070,15 +2067,15 @@ __global__ void __maxnreg__(96) wc_tc32_kernel(TcArgs A) {
         uint32_t tcount = 0;
         bool stop = false;
         for (int r = 0; !stop; ++r) {
-            const int brick = live_brick(A, G, cta, r);
-            if (brick < 0) break;
+            const int unit = live_unit(A, cta, r);
+            if (unit < 0) break;
             int r_next = r + 1;
-            const int next_brick = live_brick(A, G, cta, r_next);
+            const int next_unit = live_unit(A, cta, r_next);
             uint32_t am = 0u;
-            for (int i = 4 * A.brick_tile_ptr[brick] + lane; i < 4 * A.brick_tile_ptr[brick + 1]; i += 32)
+            for (int i = 4 * A.u_t0[unit] + lane; i < 4 * A.u_t1[unit]; i += 32)
                 am = max(am, A.tile_amax[i]);
             const float rs = ldexpf(1.0f, f16_scale_exp(warp_max_u32(am)));
-            for (int t = A.brick_tile_ptr[brick]; t < A.brick_tile_ptr[brick + 1]; ++t) {
+            for (int t = A.u_t0[unit]; t < A.u_t1[unit]; ++t) {
                 const uint32_t rb = A.rbufs == 2 ? (tcount & 1u) : 0u, rk = A.rbufs == 2 ? (tcount >> 1) : tcount;
                 unsigned char* Rb = Rs + rb * r_bytes;
                 if (tv != t) load_r_voxels(A, t, lt, RU, vv);
@@ -2101,14 +2098,14 @@ __global__ void __maxnreg__(96) wc_tc32_kernel(TcArgs A) {
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&r_full[rb]);
                 ++tcount;
-                tv = t + 1 < A.brick_tile_ptr[brick + 1] ? t + 1 : next_brick >= 0 ? A.brick_tile_ptr[next_brick] : t;
+                tv = t + 1 < A.u_t1[unit] ? t + 1 : next_unit >= 0 ? A.u_t0[next_unit] : t;
                 load_r_voxels(A, tv, lt, RU, vv);  // of the tile after this one
                 // pull the voxel rows of r of the tile A.rbufs ahead into L2
                 int tn = t + A.rbufs;
-                if (tn >= A.brick_tile_ptr[brick + 1]) {
-                    tn -= A.brick_tile_ptr[brick + 1];
-                    tn = (next_brick >= 0 && A.brick_tile_ptr[next_brick] + tn < A.brick_tile_ptr[next_brick + 1])
-                             ? A.brick_tile_ptr[next_brick] + tn : -1;
+                if (tn >= A.u_t1[unit]) {
+                    tn -= A.u_t1[unit];
+                    tn = (next_unit >= 0 && A.u_t0[next_unit] + tn < A.u_t1[next_unit])
+                             ? A.u_t0[next_unit] + tn : -1;
                 }
                 if (tn >= 0) {
                     const int32_t* tvn = A.tile_vox + (int64_t)tn * TILE_V;
@@ -2137,9 +2134,9 @@ __global__ void __maxnreg__(96) wc_tc32_kernel(TcArgs A) {
         }
         tc_fence_after();
         for (int r = 0; !stop; ++r) {
-            const int brick = live_brick(A, G, cta, r);
-            if (brick < 0) break;
-            for (int t = A.brick_tile_ptr[brick]; t < A.brick_tile_ptr[brick + 1] && !stop; ++t) {
+            const int unit = live_unit(A, cta, r);
+            if (unit < 0) break;
+            for (int t = A.u_t0[unit]; t < A.u_t1[unit] && !stop; ++t) {
                 const uint32_t rb = A.rbufs == 2 ? (tcount & 1u) : 0u, rk = A.rbufs == 2 ? (tcount >> 1) : tcount;
                 const uint32_t sR = sR0 + rb * r_bytes;
                 if (!mbar_wait(&r_full[rb], rk & 1u, &abort_flag, WAIT_LIMIT)) {
@@ -2215,7 +2212,11 @@ static TcArgs make_args(life_index_s* ix) {
     A.brick_tile_ptr = L.brick_tile_ptr.as<int32_t>();
     A.brick_fasc_ptr = L.brick_fasc_ptr.as<int32_t>();
     A.brick_fasc = L.brick_fasc.as<int32_t>();
-    A.brick_order = L.brick_order.as<int32_t>();
+    const int32_t* u = L.units.as<int32_t>();
+    A.cta_unit = u;
+    A.u_brick = u + L.grid + 1;
+    A.u_t0 = A.u_brick + L.n_units;
+    A.u_t1 = A.u_t0 + L.n_units;
     A.soff = L.soff.as<uint16_t>();
     A.wkey = L.wkey.as<uint16_t>();
     A.wfl = L.wfl.as<uint16_t>();
@@ -2315,7 +2316,7 @@ life_status dsc_tc(life_index_s* ix, const float* D, const float* w, const float
     A.n_dblk = P.n_dblk;
     auto kern = f32 ? dsc_tc_kernel<true> : dsc_tc_kernel<false>;
     LIFE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const int grid = (int)std::min<int64_t>(ix->num_sms, L.n_bricks);
+    const int grid = L.grid;
     if (n_partial) *n_partial = grid;
     if (!sparse) {
         kern<<<grid, DSC_THREADS, smem, s>>>(A);
@@ -2401,8 +2402,7 @@ life_status wc_tc(life_index_s* ix, const float* D, const float* r, float* g, co
         wc_amax_kernel<<<(unsigned)(P.n_dblk + blk), AMAX_THREADS, 0, s>>>(A, P);
         LIFE_CHECK_LAUNCH();
     }
-    const int grid = (int)std::min<int64_t>(ix->num_sms, ix->tile.n_bricks);
-    kern<<<grid, WC_THREADS, smem, s>>>(A);
+    kern<<<ix->tile.grid, WC_THREADS, smem, s>>>(A);
     LIFE_CHECK_LAUNCH();
     return LIFE_OK;
 }
