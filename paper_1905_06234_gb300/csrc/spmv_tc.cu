@@ -389,6 +389,8 @@ struct TcArgs {
     uint32_t* status;
     int nt, na, np, kp, n_sub, n_bricks, max_fb;
     int vec4;            // y / b / r pointers 16-byte aligned and Nθ % 4 == 0
+    int dstage;          // DSC, small-table form: S stages
+    int y_tile;          // DSC: the small-table form, b and Y pass through a tile in shared memory (needs vec4)
     int wgroups;         // WC: scatter warps per TMEM lane quarter (4, or 2 when shared memory is short)
     int rbufs;           // WC: R tile buffers (2 when shared memory allows: the loader runs a tile ahead)
     BatchGate bg;        // batched launch: bricks of problems that are not live are skipped, and DSC
@@ -523,7 +525,8 @@ constexpr int DSC_EPI_WARPS = 4;
 constexpr int DSC_MMA_WARP = DSC_PROD_WARPS + DSC_EPI_WARPS;
 constexpr int DSC_THREADS = (DSC_MMA_WARP + 1) * 32;
 constexpr int DSC_PROD_THREADS = DSC_PROD_WARPS * 32;
-constexpr int DSTAGE = 2;                                 // S-chunk ring depth
+constexpr int DSTAGE = 2;                                 // S-chunk ring depth, and the deepest the
+constexpr int DSTAGE_MAX = 4;                             // small-table form takes
 constexpr uint32_t DS_BYTES = TILE_V * DKC * 2;           // one S chunk: 128 rows x 128 atoms, bf16
 constexpr uint32_t DS_SBO = (DKC / 8) * 128;              // 8-row group stride of an S chunk
 
@@ -538,11 +541,15 @@ constexpr uint32_t DSC_TW = 33;  // row stride (floats) of an epilogue warp's tr
 // Shared memory of a DSC CTA: D as an MMA operand (BF16 storage only: with FP32
 // storage D's two FP16 parts sit in tensor memory), the S stages (FP32 storage:
 // hi and lo parts), the brick weight table, and (FP32) the epilogue's transpose tiles.
-__host__ __device__ inline uint32_t dsc_smem_bytes(int np, int kp, int max_fb, bool f32) {
+// (y_tile: a whole tile of Y instead, rows of dsc_y_stride bytes).
+__host__ __device__ inline uint32_t dsc_y_stride(int nt) { return (uint32_t)((nt + 31) / 32 * 32 + 4) * 4u; }
+
+__host__ __device__ inline uint32_t dsc_smem_bytes(int np, int kp, int nt, int max_fb, bool f32, int stages,
+                                                   bool y_tile) {
     uint32_t d = f32 ? 0u : (uint32_t)np * kp * 2;
     d = (d + 1023) / 1024 * 1024;
-    return d + DSTAGE * DS_BYTES * (f32 ? 2u : 1u) + 4u * (uint32_t)((max_fb + 3) / 4 * 4 + 4) +
-           (f32 ? 4u * DSC_EPI_WARPS * 32u * DSC_TW : 0u) + 1024;
+    return d + (uint32_t)stages * DS_BYTES * (f32 ? 2u : 1u) + 4u * (uint32_t)((max_fb + 3) / 4 * 4 + 4) +
+           (y_tile ? TILE_V * dsc_y_stride(nt) : f32 ? 4u * DSC_EPI_WARPS * 32u * DSC_TW : 0u) + 1024;
 }
 
 // Tensor-memory columns of a DSC CTA: two 128-column accumulators (BF16 storage),
@@ -803,17 +810,36 @@ __global__ void __launch_bounds__(PREP_THREADS) tc_prep_kernel(PrepArgs P) {
 // operand in tensor memory (lane θ), S = S_hi + S_lo the B operand in shared
 // memory, Y[θ x rows] = D_hi·S_hi + D_hi·S_lo + D_lo·S_hi in one accumulator
 // (the dropped D_lo·S_lo is ~2^-22 of the product).
-template <bool F32>
+//
+// SMALL (BF16 storage): the form for small brick tables, i.e. sparse tiles (17 entries a
+// voxel on the 64^3 workload, where a 128-atom chunk is three 256-entry blocks).  There
+// a chunk's cost is its latency, and the table leaves shared memory for more:
+//  - the tile's rows of b are bulk-copied into shared memory while its S is formed, b
+//    is subtracted from Y in place there and Y bulk-copied out: the epilogue's reads of
+//    b, a few 16-byte loads a thread at a time, took 7 us of the 8 us a tile had;
+//  - up to four S stages as they fit, and the warp that takes a chunk's first block
+//    moves on by DSC_ROT from chunk to chunk (the same three of the 23 producers had
+//    all the work).
+// 64^3 workload: 130 -> 108 us with b, an iteration 418 -> 367 us.  It is
+// taken where the tile of Y fits beside two stages: with tables of the paper's size it
+// does not, and there the tiles are dense, the producers bound the kernel, and a third
+// stage alone only costs (one-third paper workload 112 -> 127 us).  FP32 storage, whose
+// accumulator has θ along the lanes, lost by it (64^3: 176 -> 306 us).
+constexpr int DSC_ROT = 7;
+
+template <bool F32, bool SMALL>
 __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
     using SlotT = typename std::conditional<F32, EntrySlot32, EntrySlot>::type;
     constexpr uint32_t STG = F32 ? 2 * DS_BYTES : DS_BYTES;  // bytes of one S stage
     constexpr uint32_t NACC = F32 ? 1 : 2;                    // accumulators in flight
     extern __shared__ unsigned char smem_raw[];
-    __shared__ uint64_t full_bar[DSTAGE], empty_bar[DSTAGE], zero_bar[DSTAGE], acc_full[2], acc_empty[2], fin_bar,
-        tab_bar, d_ready;
+    constexpr int NST = SMALL ? DSTAGE_MAX : DSTAGE;
+    const int dst = SMALL ? A.dstage : DSTAGE;
+    __shared__ uint64_t full_bar[NST], empty_bar[NST], zero_bar[NST], acc_full[2], acc_empty[2], fin_bar, tab_bar,
+        d_ready, b_full[DSC_EPI_WARPS];
     __shared__ uint32_t tmem_base;
     __shared__ int abort_flag, never;
-    __shared__ int chunk_next[DSTAGE];  // next dynamically handed-out 256-entry block of the stage's chunk
+    __shared__ int chunk_next[NST];  // next dynamically handed-out 256-entry block of the stage's chunk
     __shared__ double red[DSC_EPI_WARPS];
     if (!A.bg.live && gate_skip(A.gate, A.gate_mode)) return;
     // full or compacted stream: of the two launches of a call, the one not chosen returns here
@@ -826,12 +852,13 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
     const uint32_t d_bytes = F32 ? 0u : align_up((uint32_t)A.np * A.kp * 2, 1024);
     unsigned char* Ds = smem;
     unsigned char* Ss = smem + d_bytes;
-    float* wl = reinterpret_cast<float*>(Ss + DSTAGE * STG);
-    float* Ts = wl + ((A.max_fb + 3) / 4 * 4 + 4);  // F32: the epilogue warps' transpose tiles
+    float* wl = reinterpret_cast<float*>(Ss + dst * STG);
+    // the epilogue warps' transpose tiles (F32), or the tile of Y (SMALL)
+    float* Ts = wl + ((A.max_fb + 3) / 4 * 4 + 4);
     const uint32_t SBO_D = (uint32_t)(A.kp / 8) * 128u;
     const uint32_t d_copy = (uint32_t)A.np * A.kp * 2;
     if (tid == 0) {
-        for (int s = 0; s < DSTAGE; ++s) {
+        for (int s = 0; s < dst; ++s) {
             mbar_init(&full_bar[s], DSC_PROD_WARPS);
             mbar_init(&empty_bar[s], 1);
             mbar_init(&zero_bar[s], 1);
@@ -842,6 +869,7 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
             mbar_init(&acc_full[b], 1);
             mbar_init(&acc_empty[b], DSC_EPI_WARPS);
         }
+        for (int w = 0; w < DSC_EPI_WARPS; ++w) mbar_init(&b_full[w], 1);
         mbar_init(&fin_bar, 1);
         // BF16 storage: one bulk copy; FP32: every producer and epilogue warp stores part of D
         mbar_init(&d_ready, F32 ? DSC_MMA_WARP : 1);
@@ -916,12 +944,14 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
         if (u0 >= 0) {
             int unit = u0, t = A.u_t0[unit], c = 0;
             int beg = chunk_beg(A, t, 0, n_c), end = chunk_end(A, t, 0, n_c);
+            int vw = warp;  // the warp's place in the chunk: it takes block vw first
+            uint32_t st = 0, ph = 0;
             int base = (beg & ~7) + tid * SLOT;
             bool have = base < end;
             SlotT cur{};
             if (have) load_slot(A.soff, A, base, cur);
             bool new_brick = true, dead = false;
-            uint32_t cc = 0, tab_ph = 0, tab_n = 0;
+            uint32_t tab_ph = 0, tab_n = 0;
             for (;;) {
                 if (new_brick) {
                     // every producer is done with the previous brick's weights (and
@@ -971,7 +1001,6 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
                         ++tab_n;
                     }
                 }
-                const uint32_t st = cc % DSTAGE, ph = (cc / DSTAGE) & 1u;
                 unsigned char* S = Ss + st * STG;
                 // the stage is free and cleared once the MMA thread's bulk zero copy lands
                 if (!dead && !warp_wait(&zero_bar[st], ph, &abort_flag)) {
@@ -986,7 +1015,8 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
                     nbeg = chunk_beg(A, nt, nc, n_c);
                     nend = chunk_end(A, nt, nc, n_c);
                 }
-                const int nbase = (nbeg & ~7) + tid * SLOT;
+                const int nvw = !SMALL ? warp : vw >= DSC_ROT ? vw - DSC_ROT : vw + DSC_PROD_WARPS - DSC_ROT;
+                const int nbase = (nbeg & ~7) + (32 * nvw + lane) * SLOT;
                 const bool nhave = nvalid && nbase < nend;
                 SlotT nxt{};
                 bool pf = false;
@@ -995,7 +1025,7 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
                 // the warps finish a chunk together.  Every lane of a warp runs the
                 // same number of slot steps, so dsc_slot can shuffle.
                 const int bb = beg & ~7;
-                int blk = warp;
+                int blk = vw;
                 while (!dead && bb + blk * (32 * SLOT) < end) {
                     int nb = 0;
                     if (lane == 0) nb = atomicAdd(&chunk_next[st], 1);
@@ -1019,8 +1049,12 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0 && !dead) mbar_arrive(&full_bar[st]);
-                ++cc;
+                if (++st == (uint32_t)dst) {
+                    st = 0;
+                    ph ^= 1u;
+                }
                 if (!nvalid) break;
+                vw = nvw;
                 r = nr;
                 unit = nunit;
                 t = nt;
@@ -1042,6 +1076,9 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
         const bool vec = A.vec4 != 0;
         uint32_t tcount = 0;
         bool stop = false;
+        // SMALL: this thread's row of the tile of Y, and the phase of its warp's b copies
+        unsigned char* yrow = reinterpret_cast<unsigned char*>(Ts) + (uint32_t)row * dsc_y_stride(A.nt);
+        uint32_t bph = 0;
         int cur_p = -1;  // batched launch: problem whose Σ out² is being accumulated
         if (A.bg.live && lane == 0 && A.partial)
             for (int p = 0; p < A.bg.n; ++p) A.partial[((int64_t)p * G + cta) * DSC_EPI_WARPS + q] = 0.0;
@@ -1059,8 +1096,20 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
             }
             for (int t = A.u_t0[unit]; t < A.u_t1[unit]; ++t) {
                 const uint32_t ab = tcount % NACC, aph = (tcount / NACC) & 1u;
-                int vj[4];  // F32: voxel of tile row 32·g + lane
-                if constexpr (F32) {
+                int vj[4];     // F32: voxel of tile row 32·g + lane
+                int vrow = -1; // SMALL: voxel of this thread's row
+                if (SMALL) {
+                    vrow = A.tile_vox[(int64_t)t * TILE_V + row];
+                    bulk_wait_all<true>();  // this lane's row of the tile before has been read out
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (A.b) {
+                        const uint32_t nv = __popc(__ballot_sync(0xffffffffu, vrow >= 0));
+                        if (lane == 0) mbar_arrive_expect_tx(&b_full[q], nv * 4u * (uint32_t)A.nt);
+                        __syncwarp();
+                        if (vrow >= 0) bulk_copy_g2s(yrow, A.b + (int64_t)A.nt * vrow, 4u * (uint32_t)A.nt, &b_full[q]);
+                    }
+                } else if constexpr (F32) {
                     // before the accumulator is ready: the tile's voxels, and its rows of b
                     // into L2 (this thread's row), so that the loads below hit L2
 #pragma unroll
@@ -1069,12 +1118,59 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
                     if (A.b && vr >= 0)
                         for (int k = 0; k < A.nt; k += 32) prefetch_l2(A.b + (int64_t)A.nt * vr + k);
                 }
-                if (!warp_wait(&acc_full[ab], aph, &abort_flag)) {
+                bool ok = warp_wait(&acc_full[ab], aph, &abort_flag);
+                if (SMALL && A.b) {  // (also before giving up: the copies are into this CTA)
+                    ok = warp_wait(&b_full[q], bph, &never) && ok;
+                    bph ^= 1u;
+                }
+                if (!ok) {
                     abort_flag = 1;
                     stop = true;
                     break;
                 }
                 tc_fence_after();
+                if (SMALL) {
+                    __syncwarp();
+                    const uint32_t taddr = tb + ((uint32_t)(32 * q) << 16) + ab * 128u;
+                    float sqf = 0.0f;
+                    uint32_t am = 0u;  // bits of max |y| over this warp's rows (for a WC of y)
+                    for (int j = 0; j < A.np; j += 16) {
+                        uint32_t rr[16];
+                        tmem_ld16(taddr + j, rr);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int e = 0; e < 16; e += 4) {
+                            if (vrow < 0 || j + e >= A.nt) continue;
+                            float4 yv = make_float4(__uint_as_float(rr[e]) * y_unscale, __uint_as_float(rr[e + 1]) * y_unscale,
+                                                    __uint_as_float(rr[e + 2]) * y_unscale, __uint_as_float(rr[e + 3]) * y_unscale);
+                            float4* cell = reinterpret_cast<float4*>(yrow) + (j + e) / 4;
+                            if (A.b) {
+                                const float4 bv = *cell;
+                                yv.x -= bv.x;
+                                yv.y -= bv.y;
+                                yv.z -= bv.z;
+                                yv.w -= bv.w;
+                            }
+                            if (wy) *cell = yv;
+                            sqf += yv.x * yv.x + yv.y * yv.y + yv.z * yv.z + yv.w * yv.w;
+                            am = max(max(am, max(abs_bits(yv.x), abs_bits(yv.y))), max(abs_bits(yv.z), abs_bits(yv.w)));
+                        }
+                        __syncwarp();
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&acc_empty[ab]);
+                    if (wy) {
+                        fence_proxy_async_smem();
+                        if (vrow >= 0) bulk_copy_s2g(A.out + (int64_t)A.nt * vrow, yrow, 4u * (uint32_t)A.nt);
+                        bulk_commit();
+                        am = warp_max_u32(am);
+                        if (lane == 0) A.tile_amax[(int64_t)t * 4 + q] = am;
+                    }
+                    sq += (double)sqf;
+                    ++tcount;
+                    continue;
+                }
                 if constexpr (F32) {
                     // Y[θ, tile row]: each 32 x 32 block (this warp's θ quarter, 32 tile
                     // rows) goes through the warp's shared-memory tile, transposed, so that
@@ -1215,6 +1311,7 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
                 ++tcount;
             }
         }
+        if (SMALL) bulk_wait_all<false>();
         if (A.bg.live) {
             if (cur_p >= 0) dsc_flush_sq(A, sq, cur_p, G, cta, q, lane);
         } else {
@@ -1225,10 +1322,10 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
         // ---------------- MMA issuer: Y[128 x 128] = D[θ x kp] · S (FP16 hi/lo operands)
         const uint32_t idesc = idesc_f16_f32(128, TILE_V);
         const uint32_t sS = smem_u32(Ss), half = (uint32_t)A.kp / 2, acc = tb + (uint32_t)A.kp;
-        uint32_t cc = 0, tcount = 0;
+        uint32_t st = 0, ph = 0, tcount = 0;
         uint32_t zlast = 0;  // bit z: parity of the last zero-copy phase issued on stage z
         bool stop = false;
-        for (int z = 0; z < DSTAGE; ++z) {  // clear both stages (hi and lo parts) for their first use
+        for (int z = 0; z < dst; ++z) {  // clear both stages (hi and lo parts) for their first use
             mbar_arrive_expect_tx(&zero_bar[z], STG);
             bulk_copy_g2s(Ss + z * STG, g_zero_chunk, DS_BYTES, &zero_bar[z]);
             bulk_copy_g2s(Ss + z * STG + DS_BYTES, g_zero_chunk, DS_BYTES, &zero_bar[z]);
@@ -1250,7 +1347,6 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
                 }
                 tc_fence_after();
                 for (int c = 0; c < n_c; ++c) {
-                    const uint32_t st = cc % DSTAGE, ph = (cc / DSTAGE) & 1u;
                     if (!mbar_wait(&full_bar[st], ph, &abort_flag, WAIT_LIMIT)) { abort_flag = 1; stop = true; break; }
                     tc_fence_after();
                     const uint32_t sb = sS + st * STG;
@@ -1271,7 +1367,10 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
                     bulk_copy_g2s(Ss + st * STG, g_zero_chunk, DS_BYTES, &zero_bar[st]);
                     bulk_copy_g2s(Ss + st * STG + DS_BYTES, g_zero_chunk, DS_BYTES, &zero_bar[st]);
                     zlast ^= 1u << st;
-                    ++cc;
+                    if (++st == (uint32_t)dst) {
+                        st = 0;
+                        ph ^= 1u;
+                    }
                 }
                 if (stop) break;
                 mma_commit(&acc_full[0]);
@@ -1280,16 +1379,16 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
         }
         mma_commit(&fin_bar);
         if (!mbar_wait(&fin_bar, 0, &never, WAIT_LIMIT)) abort_flag = 1;
-        for (int z = 0; z < DSTAGE; ++z)
+        for (int z = 0; z < dst; ++z)
             if (!mbar_wait(&zero_bar[z], (zlast >> z) & 1u, &never, WAIT_LIMIT)) abort_flag = 1;
     } else if (!F32 && lane == 0) {
         // ---------------- MMA issuer: Yᵀ[128 x np] = S[128 x kp] · Dᵀ (FP16 operands)
         const uint32_t idesc = idesc_f16_f32(128, (uint32_t)A.np);
         const uint32_t sS = smem_u32(Ss), sD = smem_u32(Ds);
-        uint32_t cc = 0, tcount = 0;
+        uint32_t st = 0, ph = 0, tcount = 0;
         uint32_t zlast = 0;  // bit z: parity of the last zero-copy phase issued on stage z
         bool stop = false;
-        for (int z = 0; z < DSTAGE; ++z) {  // clear both stages for their first use
+        for (int z = 0; z < dst; ++z) {  // clear both stages for their first use
             mbar_arrive_expect_tx(&zero_bar[z], DS_BYTES);
             bulk_copy_g2s(Ss + z * DS_BYTES, g_zero_chunk, DS_BYTES, &zero_bar[z]);
         }
@@ -1306,7 +1405,6 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
                 tc_fence_after();
                 const uint32_t d = tb + ab * 128u;
                 for (int c = 0; c < n_c; ++c) {
-                    const uint32_t st = cc % DSTAGE, ph = (cc / DSTAGE) & 1u;
                     if (!mbar_wait(&full_bar[st], ph, &abort_flag, WAIT_LIMIT)) { abort_flag = 1; stop = true; break; }
                     tc_fence_after();
 #pragma unroll
@@ -1322,7 +1420,10 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
                     mbar_arrive_expect_tx(&zero_bar[st], DS_BYTES);
                     bulk_copy_g2s(Ss + st * DS_BYTES, g_zero_chunk, DS_BYTES, &zero_bar[st]);
                     zlast ^= 1u << st;
-                    ++cc;
+                    if (++st == (uint32_t)dst) {
+                        st = 0;
+                        ph ^= 1u;
+                    }
                 }
                 if (stop) break;
                 mma_commit(&acc_full[ab]);
@@ -1333,7 +1434,7 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
         // a wait that gives up marks the call failed (the host sees LIFE_ETIMEOUT)
         if (!mbar_wait(&fin_bar, 0, &never, WAIT_LIMIT)) abort_flag = 1;
         // no bulk copy may still be writing shared memory when the CTA exits
-        for (int z = 0; z < DSTAGE; ++z)
+        for (int z = 0; z < dst; ++z)
             if (!mbar_wait(&zero_bar[z], (zlast >> z) & 1u, &never, WAIT_LIMIT)) abort_flag = 1;
     }
     tc_fence_before();
@@ -1616,13 +1717,15 @@ __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
             if (unit < 0) break;
             const int brick = A.u_brick[unit];
             const int fb0 = A.brick_fasc_ptr[brick], nfb = A.brick_fasc_ptr[brick + 1] - fb0;
+            // (The maximum is the whole brick's in every unit of it, so that the table's unit,
+            // and with it the rounding, does not depend on how bricks are shared out.)
             // Fixed point: every entry adds val·Z with |val·Z| <= max|val|·max_a Σθ|D|·max|r|
             // (up to the BF16 roundings of r and D, < 1 %), and a fascicle has at most
             // cnt entries in the brick, so |any partial sum| <= cv·d1·rmax = bnd.  With
             // sc = 2^(29 - e), bnd < 2^e, a table word stays below 2^29·1.01 + cnt/2 < 2^31.
             // Non-finite or tiny bounds keep the FP32 table.
             uint32_t am = 0u;
-            for (int i = 4 * A.u_t0[unit] + lane; i < 4 * A.u_t1[unit]; i += 32)
+            for (int i = 4 * A.brick_tile_ptr[brick] + lane; i < 4 * A.brick_tile_ptr[brick + 1]; i += 32)
                 am = max(am, A.tile_amax[i]);
             for (int o = 16; o > 0; o >>= 1) am = max(am, __shfl_xor_sync(0xffffffffu, am, o));
             const float bnd = A.brick_cv[brick] * d1 * __uint_as_float(am);
@@ -1748,9 +1851,9 @@ __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
             const int unit = live_unit(A, cta, r);
             if (unit < 0) break;
             int r_next = r + 1;
-            const int next_unit = live_unit(A, cta, r_next);
+            const int next_unit = live_unit(A, cta, r_next), brick = A.u_brick[unit];
             uint32_t am = 0u;
-            for (int i = 4 * A.u_t0[unit] + lane; i < 4 * A.u_t1[unit]; i += 32)
+            for (int i = 4 * A.brick_tile_ptr[brick] + lane; i < 4 * A.brick_tile_ptr[brick + 1]; i += 32)
                 am = max(am, A.tile_amax[i]);
             const float rs = ldexpf(1.0f, f16_scale_exp(warp_max_u32(am)));
             for (int t = A.u_t0[unit]; t < A.u_t1[unit]; ++t) {
@@ -1999,7 +2102,7 @@ __global__ void __maxnreg__(96) wc_tc32_kernel(TcArgs A) {
             const int brick = A.u_brick[unit];
             const int fb0 = A.brick_fasc_ptr[brick], nfb = A.brick_fasc_ptr[brick + 1] - fb0;
             uint32_t am = 0u;
-            for (int i = 4 * A.u_t0[unit] + lane; i < 4 * A.u_t1[unit]; i += 32)
+            for (int i = 4 * A.brick_tile_ptr[brick] + lane; i < 4 * A.brick_tile_ptr[brick + 1]; i += 32)
                 am = max(am, A.tile_amax[i]);
             am = warp_max_u32(am);
             // Z in tensor memory is 2^(kR + kD)·Z (kR from the brick's max |r|, as the loader scales R)
@@ -2070,9 +2173,9 @@ __global__ void __maxnreg__(96) wc_tc32_kernel(TcArgs A) {
             const int unit = live_unit(A, cta, r);
             if (unit < 0) break;
             int r_next = r + 1;
-            const int next_unit = live_unit(A, cta, r_next);
+            const int next_unit = live_unit(A, cta, r_next), brick = A.u_brick[unit];
             uint32_t am = 0u;
-            for (int i = 4 * A.u_t0[unit] + lane; i < 4 * A.u_t1[unit]; i += 32)
+            for (int i = 4 * A.brick_tile_ptr[brick] + lane; i < 4 * A.brick_tile_ptr[brick + 1]; i += 32)
                 am = max(am, A.tile_amax[i]);
             const float rs = ldexpf(1.0f, f16_scale_exp(warp_max_u32(am)));
             for (int t = A.u_t0[unit]; t < A.u_t1[unit]; ++t) {
@@ -2284,7 +2387,17 @@ life_status dsc_tc(life_index_s* ix, const float* D, const float* w, const float
         A.val = nullptr;
         A.val32 = L.val.as<float>();
     }
-    const uint32_t smem = dsc_smem_bytes(A.np, A.kp, A.max_fb, f32);
+    // the small-table form where a tile of Y fits beside the table, with as many S stages
+    // as fit then
+    int optin = 0;
+    LIFE_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ix->device));
+    auto fits = [&](int stages, bool y_tile) {
+        return dsc_smem_bytes(A.np, A.kp, A.nt, A.max_fb, f32, stages, y_tile) + 512 <= (uint32_t)optin;
+    };
+    A.y_tile = !f32 && A.vec4 && fits(DSTAGE, true) ? 1 : 0;
+    A.dstage = DSTAGE;
+    while (A.y_tile && A.dstage < DSTAGE_MAX && fits(A.dstage + 1, true)) ++A.dstage;
+    const uint32_t smem = dsc_smem_bytes(A.np, A.kp, A.nt, A.max_fb, f32, A.dstage, A.y_tile != 0);
     const bool sparse = L.sparse && !bg.live && L.wb_total > 0 && L.n_nnz > 0;
     if (sparse) {
         // the last block decides: full or compacted stream, rebuild or not (the
@@ -2314,7 +2427,7 @@ life_status dsc_tc(life_index_s* ix, const float* D, const float* w, const float
     A.d_img = P.img_dsc;
     A.d_info = P.info;
     A.n_dblk = P.n_dblk;
-    auto kern = f32 ? dsc_tc_kernel<true> : dsc_tc_kernel<false>;
+    auto kern = f32 ? dsc_tc_kernel<true, false> : A.y_tile ? dsc_tc_kernel<false, true> : dsc_tc_kernel<false, false>;
     LIFE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int grid = L.grid;
     if (n_partial) *n_partial = grid;
@@ -2349,14 +2462,14 @@ life_status dsc_tc(life_index_s* ix, const float* D, const float* w, const float
     }
     A.ctl = ctl;
     A.want_mode = DSC_MODE_FULL;
-    dsc_tc_kernel<false><<<grid, DSC_THREADS, smem, s>>>(A);
+    kern<<<grid, DSC_THREADS, smem, s>>>(A);
     LIFE_CHECK_LAUNCH();
     A.want_mode = DSC_MODE_COMPACT;
     A.soff = L.c_soff.as<uint16_t>();
     A.fl = L.c_fl.as<uint16_t>();
     A.val = L.c_val.as<__nv_bfloat16>();
     A.chunk_end = L.c_chunk_end.as<int32_t>();
-    dsc_tc_kernel<false><<<grid, DSC_THREADS, smem, s>>>(A);
+    kern<<<grid, DSC_THREADS, smem, s>>>(A);
     LIFE_CHECK_LAUNCH();
     return LIFE_OK;
 }
