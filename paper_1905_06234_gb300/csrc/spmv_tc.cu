@@ -1523,6 +1523,63 @@ __device__ __forceinline__ void wc_load_slot(const TcArgs& A, int base, EntrySlo
     s.val = __ldg(reinterpret_cast<const uint4*>(A.wval) + (base >> 3));
 }
 
+// A thin segment (at most WC_THIN entries; 45 on the 64^3 workload, 575 at the paper's
+// density) is taken one entry a lane, up to four times, instead of eight consecutive
+// entries a lane: with 45 entries that kept six lanes busy for eight entries each.
+// Lane i's entries beg + i, beg + 32 + i, ... sit in the four words of each field.
+// The kernels come with this path (THIN) and without: it takes WC from 135 to 114 us
+// (FP32 storage 188 to 154) on the 64^3 workload, and at the paper's density, where no
+// segment is thin, costs 5 % (294 to 309 us).  A launch takes it when its segments hold
+// at most WC_THIN_MEAN entries on average (64^3 grids: at 91 a segment 122 against 138
+// us, FP32 166 against 199; at 136, where most are no longer thin, 160 against 154).
+constexpr int WC_THIN = 128;
+constexpr int WC_THIN_MEAN = 96;
+
+__device__ __forceinline__ void wc_load_thin(const TcArgs& A, int beg, int end, int lane, uint32_t (&key)[4],
+                                             uint32_t (&fl)[4]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int j = beg + 32 * i + lane;
+        key[i] = j < end ? (uint32_t)__ldg(A.wkey + j) : 0u;
+        fl[i] = j < end ? (uint32_t)__ldg(A.wfl + j) : 0u;
+    }
+}
+
+template <bool FIXED>
+__device__ __forceinline__ void wc_thin(const uint32_t (&key)[4], const uint32_t (&fl)[4], const float (&val)[4], int beg,
+                                        int end, int lane, const float* Zw, float* gl, uint32_t gl_s) {
+    float x[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        if (beg + 32 * i < end) x[i] = val[i] * *reinterpret_cast<const float*>(reinterpret_cast<const char*>(Zw) + key[i]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (beg + 32 * i + lane >= end) continue;
+        if (FIXED) atomicAdd(reinterpret_cast<int*>(reinterpret_cast<char*>(gl) + fl[i]), __float2int_rn(x[i]));
+        else red_add_shared_f32(gl_s + fl[i], x[i]);
+    }
+}
+
+// The first entries of a segment: a thin one's all, else the first two blocks' slots.
+template <bool THIN>
+__device__ __forceinline__ void wc_load_first(const TcArgs& A, int beg, int end, int lane, EntrySlot& s0, EntrySlot& s1) {
+    if (THIN && end - beg <= WC_THIN) {
+        uint32_t k[4], f[4];
+        wc_load_thin(A, beg, end, lane, k, f);
+        s0.key = make_uint4(k[0], k[1], k[2], k[3]);
+        s0.fl = make_uint4(f[0], f[1], f[2], f[3]);
+        const uint16_t* wv = reinterpret_cast<const uint16_t*>(A.wval) + beg + lane;
+        s0.val.x = beg + lane < end ? (uint32_t)__ldg(wv) << 16 : 0u;
+        s0.val.y = beg + 32 + lane < end ? (uint32_t)__ldg(wv + 32) << 16 : 0u;
+        s0.val.z = beg + 64 + lane < end ? (uint32_t)__ldg(wv + 64) << 16 : 0u;
+        s0.val.w = beg + 96 + lane < end ? (uint32_t)__ldg(wv + 96) << 16 : 0u;
+        return;
+    }
+    const int base = (beg & ~7) + lane * SLOT;
+    if (base < end) wc_load_slot(A, base, s0);
+    if (base + 32 * SLOT < end) wc_load_slot(A, base + 32 * SLOT, s1);
+}
+
 __device__ __forceinline__ int wseg(const TcArgs& A, int t, int q, int s) {
     return A.wseg_ptr[((int64_t)t * 4 + q) * A.n_sub + s];
 }
@@ -1651,6 +1708,7 @@ __device__ __forceinline__ void load_r_tile(const TcArgs& A, int t, const RUnits
     }
 }
 
+template <bool THIN>
 __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ uint64_t r_full[2], r_empty[2], z_full[ZSLOTS], z_empty[ZSLOTS], fin_bar, d_ready;
@@ -1757,8 +1815,7 @@ __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
             if (!active) beg = end = 0;
             int base = (beg & ~7) + lane * SLOT;
             EntrySlot cur0 = zero, cur1 = zero;
-            if (active && base < end) wc_load_slot(A, base, cur0);
-            if (active && base + BLK < end) wc_load_slot(A, base + BLK, cur1);
+            if (active) wc_load_first<THIN>(A, beg, end, lane, cur0, cur1);
             for (int t = t0; t < t1 && !dead; ++t) {
                 for (int j = 0; j < kc && !dead; ++j, ++kcount) {
                     // chunk j (atoms 128j ..) of tile t sits in slot zs of the ring
@@ -1790,6 +1847,15 @@ __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
 #pragma unroll
                                 for (int e = 0; e < 32; ++e) zrow[e] = __uint_as_float(rr[e]) * sc;
                                 __syncwarp();
+                                if (THIN && end - beg <= WC_THIN) {
+                                    wc_load_first<THIN>(A, nbeg, nend, lane, nxt0, nxt1);
+                                    const uint32_t k[4] = {cur0.key.x, cur0.key.y, cur0.key.z, cur0.key.w},
+                                                   f[4] = {cur0.fl.x, cur0.fl.y, cur0.fl.z, cur0.fl.w};
+                                    const float x[4] = {__uint_as_float(cur0.val.x), __uint_as_float(cur0.val.y),
+                                                        __uint_as_float(cur0.val.z), __uint_as_float(cur0.val.w)};
+                                    if (fixed) wc_thin<true>(k, f, x, beg, end, lane, Zw, gl, gl_s);
+                                    else wc_thin<false>(k, f, x, beg, end, lane, Zw, gl, gl_s);
+                                } else
                                 for (;;) {
                                     const int b2 = base + 2 * BLK;
                                     const bool more = __shfl_sync(0xffffffffu, b2, 0) < end;
@@ -1797,8 +1863,7 @@ __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
                                         if (b2 < end) wc_load_slot(A, b2, nxt0);
                                         if (b2 + BLK < end) wc_load_slot(A, b2 + BLK, nxt1);
                                     } else {
-                                        if (nbase < nend) wc_load_slot(A, nbase, nxt0);
-                                        if (nbase + BLK < nend) wc_load_slot(A, nbase + BLK, nxt1);
+                                        wc_load_first<THIN>(A, nbeg, nend, lane, nxt0, nxt1);
                                     }
                                     if (fixed) {
                                         wc_slot<true>(cur0, base, beg, end, Zw, gl, gl_s);
@@ -1816,8 +1881,7 @@ __global__ void __maxnreg__(96) wc_tc_kernel(TcArgs A) {
                                 }
                                 __syncwarp();
                             } else {
-                                if (nbase < nend) wc_load_slot(A, nbase, nxt0);
-                                if (nbase + BLK < nend) wc_load_slot(A, nbase + BLK, nxt1);
+                                wc_load_first<THIN>(A, nbeg, nend, lane, nxt0, nxt1);
                             }
                             cur0 = nxt0;
                             cur1 = nxt1;
@@ -2020,6 +2084,7 @@ __device__ __forceinline__ void wc32_segment(const TcArgs& A, int beg, int end, 
     }
 }
 
+template <bool THIN>
 __global__ void __maxnreg__(96) wc_tc32_kernel(TcArgs A) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ uint64_t r_full[2], r_empty[2], z_full[Z32_SLOTS], z_empty[Z32_SLOTS], fin_bar, d_ready;
@@ -2124,6 +2189,22 @@ __global__ void __maxnreg__(96) wc_tc32_kernel(TcArgs A) {
                     for (int hh = 0; hh < 2 && !dead; ++hh, ++kcount) {
                         // rows 64hh .. of atom block j sit in slot zs of the ring
                         const uint32_t zs = kcount % Z32_SLOTS, zu = (kcount / Z32_SLOTS) & 1u;
+                        // a thin segment's entries are on their way while its Z is waited for
+                        // (with four scatter groups a warp has one row quarter, h)
+                        uint32_t tk[4], tf[4];
+                        float tx[4];
+                        bool thin = false;
+                        if (THIN) {
+                            const int tb0 = __shfl_sync(0xffffffffu, bq[0], 4 * j + q);
+                            const int te0 = __shfl_sync(0xffffffffu, bq[0], 4 * j + q + 1);
+                            thin = (h >> 1) == hh && te0 - tb0 <= WC_THIN;  // (no entries: te0 = tb0)
+                            if (thin) {
+                                wc_load_thin(A, tb0, te0, lane, tk, tf);
+#pragma unroll
+                                for (int i = 0; i < 4; ++i)
+                                    tx[i] = tb0 + 32 * i + lane < te0 ? __ldg(A.wval32 + tb0 + 32 * i + lane) : 0.0f;
+                            }
+                        }
                         if (!warp_wait(&z_full[zs], zu, &abort_flag)) {
                             abort_flag = 1;
                             dead = true;
@@ -2147,7 +2228,8 @@ __global__ void __maxnreg__(96) wc_tc32_kernel(TcArgs A) {
 #pragma unroll
                                 for (int e = 0; e < 32; ++e) zrow[e] = __uint_as_float(rr[e]) * sc;
                                 __syncwarp();
-                                wc32_segment(A, beg, end, Zw, gl_s, lane);
+                                if (THIN && k == 0 && thin) wc_thin<false>(tk, tf, tx, beg, end, lane, Zw, gl, gl_s);
+                                else wc32_segment(A, beg, end, Zw, gl_s, lane);
                                 __syncwarp();
                             }
                         }
@@ -2501,7 +2583,8 @@ life_status wc_tc(life_index_s* ix, const float* D, const float* r, float* g, co
         A.wval32 = ix->tile.wval.as<float>();
     }
     const uint32_t smem = wc_smem_bytes(A.np, A.kp, A.max_fb, A.wgroups, A.rbufs, f32);
-    auto kern = f32 ? wc_tc32_kernel : wc_tc_kernel;
+    const bool thin = ix->nnz <= (int64_t)WC_THIN_MEAN * ix->tile.n_tiles * 4 * A.n_sub;
+    auto kern = f32 ? (thin ? wc_tc32_kernel<true> : wc_tc32_kernel<false>) : thin ? wc_tc_kernel<true> : wc_tc_kernel<false>;
     LIFE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // (blocks as in the launch that wrote d_info: the DSC's, or this call's own)
     const PrepArgs P = prep_args(ix, D, g, r_is_dsc_out ? PREP_THREADS : AMAX_THREADS);

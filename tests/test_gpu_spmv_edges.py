@@ -66,3 +66,30 @@ def test_direction_counts(life, form, nt):
                                             (20000, 9000, 8), (40000, 300000, 4), (5000, 0, 8), (2048, 200000, 16)])
 def test_tile_and_brick_counts(life, form, nv, n, brick_dim):
     check(life, form, 96, 200, nv, 3000, n, brick_dim)
+
+
+@pytest.mark.parametrize("form", ["bf16", "fp32"])
+@pytest.mark.parametrize("edge", [31, 32, 33, 64, 127, 128, 129, 256, 257, 600])
+def test_thin_and_thick_segments(life, form, edge):
+    """WC segments (32 voxels x 32 atoms) of `edge` entries and of none among thin ones."""
+    nt, na, nv, nf = 32, 96, 384, 900
+    rng = np.random.default_rng(edge)
+    n = 3000
+    a, v, f = (rng.integers(0, k, n).astype(np.int32) for k in (na, nv, nf))
+    f2 = rng.permutation(nf)[:edge].astype(np.int32)            # one segment gets exactly `edge` distinct entries
+    keep = ~((a // 32 == 1) & (v // 32 == 3))
+    a = np.concatenate([a[keep], np.full(edge, 32 + 5, np.int32)])
+    v = np.concatenate([v[keep], (96 + rng.integers(0, 32, edge)).astype(np.int32)])
+    f = np.concatenate([f[keep], f2])
+    x = rng.uniform(0.5, 1.0, len(a)).astype(np.float32)
+    D, r = (rng.standard_normal(k).astype(np.float32) for k in (nt * na, nt * nv))
+    prec = life.LIFE_BF16 if form == "bf16" else life.LIFE_FP32
+    idx = life.index_from_arrays(a, v, f, x, nt, na, nv, nf, precision=prec, algo=life.LIFE_ALGO_TC)
+    phi = oracle.canon(a, v, f, x, na, nv, nf)
+    g, _ = life.life_wc(idx, torch.from_numpy(D).cuda(), torch.from_numpy(r).cuda())
+    life.life_check_device_status()
+    g, g_ref = g.cpu().numpy(), oracle.wc(phi, D, r, nt, nf)
+    if form == "bf16":
+        assert (np.abs(g - g_ref) <= rounding_bounds(phi, D, np.zeros(nf, np.float32), r, nt, nv, nf)[1] + 1e-30).all()
+    else:
+        assert rel(g, g_ref) <= 1e-5
