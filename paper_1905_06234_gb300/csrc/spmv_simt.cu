@@ -38,12 +38,26 @@ __device__ __forceinline__ double block_sum_f64(double v, double* sh) {
     return t;  // valid in thread 0
 }
 
+// D into shared memory, columns padded to NTW·32 floats; by 16-byte accesses where D
+// allows, eight a thread in flight (one float at a time, the 138 KB of a 96 x 360 D
+// were a third of a small call's time).
 template <int NTW>
 __device__ __forceinline__ void stage_D(float* Ds, const float* __restrict__ D, int nt, int na) {
-    const int ntp = NTW * 32;
-    for (int i = threadIdx.x; i < na * ntp; i += blockDim.x) {
+    constexpr int ntp = NTW * 32;
+    if ((nt & 3) == 0 && (reinterpret_cast<uintptr_t>(D) & 15) == 0) {
+        constexpr int q = ntp / 4;
+#pragma unroll 8
+        for (int i = threadIdx.x; i < na * q; i += SIMT_THREADS) {
+            const int a = i / q, t = 4 * (i - a * q);
+            reinterpret_cast<float4*>(Ds)[i] = t < nt ? __ldg(reinterpret_cast<const float4*>(D + (int64_t)nt * a + t))
+                                                      : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
+        return;
+    }
+#pragma unroll 8
+    for (int i = threadIdx.x; i < na * ntp; i += SIMT_THREADS) {
         const int a = i / ntp, t = i - a * ntp;
-        Ds[i] = t < nt ? D[t + (int64_t)nt * a] : 0.0f;
+        Ds[i] = t < nt ? __ldg(D + t + (int64_t)nt * a) : 0.0f;
     }
 }
 
@@ -64,7 +78,7 @@ dsc_simt_kernel(const int32_t* __restrict__ vox_ptr, const uint16_t* __restrict_
                 int nt, int na, int nv, const float* __restrict__ w, const float* __restrict__ b,
                 float* __restrict__ y, double* __restrict__ partial, const life_sbb_state* gate, int gate_mode,
                 const BatchGate bg) {
-    extern __shared__ float Ds[];
+    extern __shared__ __align__(16) float Ds[];
     __shared__ double red[32];
     bool write_y = y != nullptr;
     if (!bg.live) {
