@@ -109,8 +109,8 @@ life_status exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t n, cudaS
 // A pass is bound by memory: 12 B per pair read and written, 8 B more read by the
 // histograms.  The scatter orders its tile by digit in shared memory before it
 // writes, so that a warp writes a few runs of consecutive pairs instead of 32
-// scattered ones (32-byte sectors of which 12 B were used): 8192 pairs a tile give
-// runs of 32 pairs at 8 bits, 64 at 7, and two CTAs of 512 threads share an SM.
+// scattered ones (32-byte sectors of which 12 B were used): 6144 pairs a tile give
+// runs of 24 pairs at 8 bits, 48 at 7, and two CTAs of 512 threads share an SM.
 // The index build of the paper-scale workload (80M entries, BF16 storage) took
 // 80.0 ms with 22 passes of an unstaged scatter (1.9 ms each), 44.0 ms with this
 // one, 16 passes (the callers sort only the bits that are not in order yet) and
@@ -118,8 +118,8 @@ life_status exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t n, cudaS
 
 constexpr int RS_THREADS = 512;
 constexpr int RS_WARPS = RS_THREADS / 32;
-constexpr int RS_ROUNDS = 16;                     // items per lane
-constexpr int RS_TILE = RS_THREADS * RS_ROUNDS;   // 8192 items per block
+constexpr int RS_ROUNDS = 12;                     // items per lane (16 spill; paper-scale build 14.7 ms, with 12 14.3)
+constexpr int RS_TILE = RS_THREADS * RS_ROUNDS;   // 6144 items per block
 constexpr int RS_DIGITS = 256;
 constexpr int RS_COPIES = 8;                      // histogram copies: two warps add to each
 constexpr size_t RS_SMEM = (size_t)RS_TILE * 12 + sizeof(uint16_t) * RS_WARPS * RS_DIGITS;

@@ -390,7 +390,7 @@ __global__ void wb_src_kernel(const int32_t* __restrict__ bptr, const int32_t* _
 constexpr int TS_THREADS = 1024;
 constexpr int TS_CELLS = TILE_V * DKC;                 // cells of one pass: 16 a thread
 constexpr int TS_PER = TS_CELLS / TS_THREADS;
-constexpr int TS_BATCH = 4;                            // entries whose loads a thread issues together
+constexpr int TS_BATCH = 2;                            // entries whose loads a thread issues together (4 spill)
 constexpr int TS_MAX_C = 4;                            // 128-atom chunks (Na <= 512)
 constexpr int TS_STAGE = 19456;                        // entries staged in shared memory before they are written
 constexpr size_t TS_SMEM = sizeof(int32_t) * TS_CELLS + sizeof(uint2) * TS_STAGE;
