@@ -147,11 +147,13 @@ def _ptr(t):
         raise ValueError("liblife takes CUDA tensors")
     if not t.is_contiguous():
         raise ValueError("liblife takes contiguous tensors")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()   # a plain address: the argument types make a pointer of it
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    # the raw handle: a small call (11 us on the GPU) is bound by the host, and the stream
+    # object torch.cuda.current_stream() makes is most of what this module adds to it
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _need(t, dtype, numel, name):
