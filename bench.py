@@ -33,18 +33,18 @@ PEAK_FALLBACK = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0}
 # DRAM bytes (read + write) of the launches of one timed tensor-core call, from
 # ncu captures (dram__bytes_read.sum + dram__bytes_write.sum, one kernel per
 # capture) on the paper-density workload at a third of the size: DSC with the
-# fused residual = max|w| pass + DSC kernel; WC through the public call =
-# per-tile max|r| pass + WC kernel; per path (BF16 storage, FP32 storage on the
+# fused residual = preparation launch + DSC kernel; WC through the public call =
+# max|r| and preparation launch + WC kernel; per path (BF16 storage, FP32 storage on the
 # tensor cores).  Scaled to the timed workload by its entry count (the traffic
 # grows with the entries and voxels alike).  The figures hold only for the kernel
 # source that was captured; after any change to it the bench reports null.
 TRAFFIC_CAPTURE = {
     "src": os.path.join("paper_1905_06234_gb300", "csrc", "spmv_tc.cu"),
-    "sha256": "c2ce55ecc66241ca51bf6295504ca4d5f7318b4270cc02fecf8076e9626f776a",
+    "sha256": "08e64cd0fa52498f90317c2407f4bd2e98f22266e4a9500bef050c5b7a6ed5e8",
     "nnz": 23816750,
     "bytes": {
-        "bf16-tc": {"dsc": (607488 + 0) + (197645312 + 16574976), "wc": (39993600 + 0) + (201986816 + 118016)},
-        "fp32-tc": {"dsc": (607488 + 0) + (248668160 + 20288256), "wc": (39993856 + 0) + (252520448 + 125696)},
+        "bf16-tc": {"dsc": (762112 + 0) + (197602560 + 16938240), "wc": (40148224 + 7936) + (201893376 + 47104)},
+        "fp32-tc": {"dsc": (761856 + 0) + (248656896 + 19802880), "wc": (40147968 + 0) + (256412416 + 117248)},
     },
 }
 
@@ -278,8 +278,8 @@ def e2e_steps(life, path, steps, warmup):
 
 def launches_per_step(path):
     # DSC + WC + project + scalars + DSC + WC + sumsq + scalars + update + the
-    # solve loop's condition kernel, and on the tensor-core path the brick weight
-    # gather before each of the two DSCs (the WCs take the per-tile max |r| from
+    # solve loop's condition kernel, and on the tensor-core path the preparation
+    # launch before each of the two DSCs (the WCs take the per-tile max |r| from
     # the DSC before them, so the step launches no separate max pass)
     return 12 if path.info["algo"] == 2 else 10
 
