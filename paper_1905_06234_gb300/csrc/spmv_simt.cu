@@ -623,7 +623,8 @@ graddD_chunk_kernel(const int32_t* __restrict__ chunk_beg, int n_chunks, const i
         }
         for (int base = beg; base < end; base += 32) {
             const int v = v1, k2 = base + 32 + lane;
-            float rs = s1;
+            const float s0 = s1;
+            float rs = s0;
             v1 = -1 - lane;
             s1 = 0.0f;
             if (k2 < end) {
@@ -638,19 +639,28 @@ graddD_chunk_kernel(const int32_t* __restrict__ chunk_beg, int n_chunks, const i
                 const float y2 = __shfl_up_sync(0xffffffffu, rs, o);
                 if (lane - o >= start) rs += y2;
             }
-            // no skip on a zero sum: a NaN or inf in gy must reach dL/dD as in the oracle
+            // A NaN or inf in gy must reach dL/dD as in the oracle's sum over the entries: no
+            // skip on a zero sum, and a run whose terms would differ in sign for an infinite
+            // gy (inf - inf, inf * 0) is marked by the voxel's sign bit
+            const uint32_t pos = __ballot_sync(0xffffffffu, s0 > 0.0f), neg = __ballot_sync(0xffffffffu, s0 < 0.0f),
+                           zer = __ballot_sync(0xffffffffu, s0 == 0.0f),
+                           run = (0xffffffffu >> (31 - lane)) & (0xffffffffu << start);
+            const bool mixed = ((pos & run) != 0u) + ((neg & run) != 0u) + ((zer & run) != 0u) > 1;
             const bool tail = v >= 0 && (lane == 31 || v_dn != v);
             const uint32_t m = __ballot_sync(0xffffffffu, tail);
-            if (tail) buf[__popc(m & ((1u << lane) - 1u))] = make_float2(rs, __int_as_float(v));
+            if (tail)
+                buf[__popc(m & ((1u << lane) - 1u))] = make_float2(rs, __uint_as_float((uint32_t)v | (mixed ? 0x80000000u : 0u)));
             __syncwarp();
             const int n = __popc(m);
             for (int j0 = 0; j0 < n; j0 += U) {
                 float e[U][NTW], sj[U];
+                bool mx[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const float2 x = j0 + u < n ? buf[j0 + u] : make_float2(0.0f, 0.0f);
                     sj[u] = x.x;
-                    const float* col = gy + (int64_t)nt * __float_as_int(x.y);
+                    mx[u] = __float_as_int(x.y) < 0;
+                    const float* col = gy + (int64_t)nt * (__float_as_int(x.y) & 0x7FFFFFFF);
 #pragma unroll
                     for (int q = 0; q < NTW; ++q) {
                         const int t = q * 32 + lane;
@@ -658,9 +668,13 @@ graddD_chunk_kernel(const int32_t* __restrict__ chunk_beg, int n_chunks, const i
                     }
                 }
 #pragma unroll
-                for (int u = 0; u < U; ++u)
+                for (int u = 0; u < U; ++u) {
 #pragma unroll
-                    for (int q = 0; q < NTW; ++q) acc[q] = fmaf(e[u][q], sj[u], acc[q]);
+                    for (int q = 0; q < NTW; ++q) {
+                        acc[q] = fmaf(e[u][q], sj[u], acc[q]);
+                        if (mx[u]) acc[q] = fmaf(e[u][q], 0.0f, acc[q]);  // nothing but for an infinite gy: NaN
+                    }
+                }
             }
             __syncwarp();  // the buffer is rewritten by the next window
         }
