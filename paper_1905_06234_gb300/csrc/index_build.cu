@@ -275,8 +275,9 @@ __global__ void __launch_bounds__(256) pack_vaf_kernel(const int32_t* __restrict
     const int64_t i0 = 4 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
     uint32_t bad = 0;
     if (i0 < n) {
-        int32_t a[4], v[4], f[4];
-        float x[4];
+        // (aligned: written and read 16 bytes at a time where they do not stay in registers)
+        __align__(16) int32_t a[4], v[4], f[4];
+        __align__(16) float x[4];
         const int m = (int)min((int64_t)4, n - i0);
         if (vec && m == 4) {
             *reinterpret_cast<int4*>(a) = __ldg(reinterpret_cast<const int4*>(atom + i0));
@@ -309,7 +310,9 @@ __global__ void __launch_bounds__(256) pack_vaf_kernel(const int32_t* __restrict
             *reinterpret_cast<ulonglong2*>(key + i0 + 2) = make_ulonglong2(k[2], k[3]);
             *reinterpret_cast<float4*>(payload + i0) = *reinterpret_cast<const float4*>(x);
         } else {
-            for (int e = 0; e < m; ++e) {
+#pragma unroll
+            for (int e = 0; e < 3; ++e) {  // (unrolled: the arrays stay in registers)
+                if (e >= m) break;
                 key[i0 + e] = k[e];
                 payload[i0 + e] = __float_as_uint(x[e]);
             }
