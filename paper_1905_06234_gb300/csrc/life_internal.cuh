@@ -85,10 +85,13 @@ struct TmpBuf {
     TmpBuf() = default;
     TmpBuf(const TmpBuf&) = delete;
     TmpBuf& operator=(const TmpBuf&) = delete;
-    ~TmpBuf() {
+    ~TmpBuf() { release(); }
+    void release() {
         if (p) cudaFreeAsync(p, s);
+        p = nullptr;
     }
     life_status alloc(size_t n, cudaStream_t st) {
+        release();  // (a buffer allocated again, as in a retry loop, gives its memory back first)
         s = st;
         if (n == 0) n = 16;
         cudaError_t e = cudaMallocAsync(&p, n, st);
