@@ -14,7 +14,8 @@
 // whole index build took 44.0 ms that way and takes 16.6 ms now, of which the
 // bricks' tables are 1.3 ms and the streams 3.1 ms (bound by the latency of a
 // pass: one 1024-thread CTA an SM, since a pass's cells and entries fill its
-// shared memory).  The host's part of the old build (a stable sort of the voxels,
+// shared memory).  (Sorting stays the better way for some shapes: see sort_is_faster.)
+// The host's part of the old build (a stable sort of the voxels,
 // copies both ways) went with it.
 #include <algorithm>
 #include <cstring>
@@ -159,20 +160,26 @@ __global__ void tile_fill_kernel(const uint32_t* __restrict__ vox, const int32_t
     }
 }
 
-// Entries of each tile (one warp per tile), with a zero after the last for the scan.
+// Entries of each tile (one warp per tile), with a zero after the last for the scan,
+// and of its fullest quarter of 32 rows.
 __global__ void tile_count_kernel(const int32_t* __restrict__ tile_vox, const int32_t* __restrict__ vox_ptr,
-                                  int64_t n_tiles, int32_t* __restrict__ count) {
+                                  int64_t n_tiles, int32_t* __restrict__ count, int32_t* __restrict__ quarter) {
     const int lane = threadIdx.x & 31;
     const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (t > n_tiles) return;
-    int32_t c = 0;
+    int32_t sum = 0, most = 0;
     if (t < n_tiles)
         for (int r = lane; r < TILE_V; r += 32) {
             const int32_t v = tile_vox[t * TILE_V + r];
-            if (v >= 0) c += vox_ptr[v + 1] - vox_ptr[v];
+            int32_t c = v >= 0 ? vox_ptr[v + 1] - vox_ptr[v] : 0;
+            for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+            sum += c;
+            most = max(most, c);
         }
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if (lane == 0) count[t] = c;
+    if (lane == 0) {
+        count[t] = sum;
+        quarter[t] = most;
+    }
 }
 
 // ------------------------------------------------------ brick fascicle tables
@@ -626,8 +633,150 @@ __global__ void __launch_bounds__(TS_THREADS) tile_stream_kernel(const TileStrea
     if (lane == 0 && best) atomicMax(A.vmax, best);
 }
 
-__global__ void fill_kernel(int32_t* p, int64_t n, int32_t v) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) p[i] = v;
+// ------------------------------------------------ the same layout by sorting
+//
+// Counting gives a brick and a tile one CTA each.  That is slower than sorting where
+// the entries lie in few, very full tiles (a pass of the streams walks its entries
+// once for every TS_STAGE of them), with very many fascicles (the tables walk a
+// brick's entries once for every BT_WINDOW ids) and with nearly empty tiles.  There (sort_is_faster) radix sorts of
+// (key, entry) pairs over the whole GPU take its place: by (brick, fascicle) for the
+// tables, by (tile, cell in stream order) for each stream; the list is in (v, a, f)
+// order and the sort stable, so the fascicles of a cell stay in order.  The layout is
+// the same, bit for bit.
+enum : int { BY_TABLE = 0, BY_DSC = 1, BY_WC = 2 };
+
+// tile · TILE_V + row of each voxel.
+__global__ void voxel_slot_kernel(const int32_t* __restrict__ tile_vox, int64_t n, int64_t* __restrict__ slot) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        if (tile_vox[i] >= 0) slot[tile_vox[i]] = i;
+}
+
+// Key of each entry of the merged list: brick | fascicle (bf bits), or tile | cell in the
+// order of the DSC or the WC stream (16 bits); payload = the entry.
+__global__ void entry_key_kernel(const int32_t* __restrict__ vox_ptr, int32_t nv, const int64_t* __restrict__ slot,
+                                 const int32_t* __restrict__ tile_brick, const uint16_t* __restrict__ atom,
+                                 const int32_t* __restrict__ fasc, int64_t m, int order, int bf,
+                                 uint64_t* __restrict__ key, uint32_t* __restrict__ payload) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+        int32_t lo = 0, hi = nv - 1;  // the entry's voxel: the last that starts at or before it
+        while (lo < hi) {
+            const int32_t mid = lo + (hi - lo + 1) / 2;
+            if (__ldg(vox_ptr + mid) <= i) lo = mid;
+            else hi = mid - 1;
+        }
+        const int64_t s = slot[lo], t = s / TILE_V;
+        const uint32_t row = (uint32_t)(s % TILE_V), a = atom[i];
+        key[i] = order == BY_TABLE ? ((uint64_t)tile_brick[t] << bf) | (uint64_t)fasc[i]
+                 : order == BY_DSC ? ((uint64_t)t << 16) | ((a >> 7) << 14) | dsc_cell(a, row)
+                                   : ((uint64_t)t << 16) | ((row >> 5) << 14) | (a << 5) | (row & 31u);
+        payload[i] = (uint32_t)i;
+    }
+}
+
+// Offsets of the bricks' tables from the sorted (brick, fascicle) keys.
+__global__ void sorted_bptr_kernel(const uint64_t* __restrict__ key, int64_t m, int bf, const int32_t* __restrict__ head,
+                                   const int32_t* __restrict__ uidx, int32_t nb, int32_t n_unique,
+                                   int32_t* __restrict__ bptr) {
+    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
+        if (!head[j]) continue;
+        const int32_t b = (int32_t)(key[j] >> bf), pb = j == 0 ? -1 : (int32_t)(key[j - 1] >> bf);
+        for (int32_t q = pb + 1; q <= b; ++q) bptr[q] = uidx[j];
+        if (uidx[j] == n_unique - 1)
+            for (int32_t q = b + 1; q <= nb; ++q) bptr[q] = n_unique;
+    }
+}
+
+// The tables' fascicles, the first sorted entry of each slot, and each entry's slot offset.
+__global__ void sorted_table_kernel(const uint64_t* __restrict__ key, const uint32_t* __restrict__ pay, int64_t m, int bf,
+                                    const int32_t* __restrict__ head, const int32_t* __restrict__ uidx,
+                                    const int32_t* __restrict__ bptr, int32_t* __restrict__ bfasc,
+                                    int32_t* __restrict__ first, uint16_t* __restrict__ fl) {
+    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t u = uidx[j] + head[j] - 1;  // (uidx counts the heads before j)
+        fl[pay[j]] = (uint16_t)(4 * (u - bptr[key[j] >> bf]));
+        if (head[j]) {
+            bfasc[u] = (int32_t)(key[j] & ((1ull << bf) - 1));
+            first[u] = (int32_t)j;
+        }
+    }
+}
+
+// max into p[b], one atomic where the warp has one b (almost always: the keys are sorted).
+__device__ __forceinline__ void brick_max(uint32_t* p, uint32_t b, uint32_t x) {
+    if (__all_sync(0xffffffffu, b == __shfl_sync(0xffffffffu, b, 0))) {
+        x = __reduce_max_sync(0xffffffffu, x);
+        if ((threadIdx.x & 31) == 0) atomicMax(p + b, x);
+    } else {
+        atomicMax(p + b, x);
+    }
+}
+
+// Largest entry count of a slot, and largest |val|, of each brick (both zero before).
+template <class VT>
+__global__ void sorted_cv_max_kernel(const uint64_t* __restrict__ key, const uint32_t* __restrict__ pay, int64_t m, int bf,
+                                     const int32_t* __restrict__ head, const int32_t* __restrict__ uidx,
+                                     const int32_t* __restrict__ first, int32_t n_unique, const VT* __restrict__ val,
+                                     uint32_t* __restrict__ cmax, uint32_t* __restrict__ vmax) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t j0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) - lane; j0 < m;
+         j0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t j = min(j0 + lane, m - 1);  // (lanes beyond the end repeat the last entry)
+        const uint32_t b = (uint32_t)(key[j] >> bf);
+        const int32_t u = uidx[j];
+        brick_max(cmax, b, head[j] ? (uint32_t)((u + 1 < n_unique ? (int64_t)first[u + 1] : m) - j) : 0u);
+        brick_max(vmax, b, __float_as_uint(load_val(val + pay[j])) & 0x7FFFFFFFu);
+    }
+}
+
+__global__ void sorted_cv_kernel(const uint32_t* __restrict__ cmax, const uint32_t* __restrict__ vmax, int32_t nb,
+                                 float* __restrict__ cv) {
+    for (int32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x)
+        cv[b] = __fmul_ru((float)cmax[b], __uint_as_float(vmax[b]));
+}
+
+// A stream from its sorted keys: the DSC's (WC = false: chunk offsets, continuation bits)
+// or the WC's (segment offsets); n_seg segments, the offsets one longer.
+template <class VT, bool WC>
+__global__ void sorted_stream_kernel(const uint64_t* __restrict__ key, const uint32_t* __restrict__ pay, int64_t m,
+                                     const uint16_t* __restrict__ flv, const VT* __restrict__ val, int n_c, int n_sub,
+                                     int atom_major, int64_t n_seg, uint16_t* __restrict__ okey,
+                                     uint16_t* __restrict__ ofl, VT* __restrict__ oval, int32_t* __restrict__ seg_ptr) {
+    auto seg_of = [&](uint64_t k) -> int64_t {
+        const int64_t t = (int64_t)(k >> 16), part = (int64_t)((k >> 14) & 3u);  // chunk, or row quarter
+        return WC ? (t * 4 + part) * n_sub + (int64_t)((k >> 10) & 15u) : t * n_c + part;
+    };
+    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
+        const uint64_t k = key[j];
+        const uint32_t c = (uint32_t)k & 0x3FFFu, i = pay[j];
+        if (WC) {
+            const uint32_t a32 = (c >> 5) & 31u, r32 = c & 31u;
+            okey[j] = (uint16_t)(4 * (atom_major ? a32 * ZW + r32 : r32 * ZW + a32));
+        } else {
+            const uint32_t row = ((c >> 10) << 3) | ((c >> 3) & 7u), a = (((c >> 6) & 15u) << 3) | (c & 7u);
+            okey[j] = (uint16_t)(ptx::kmajor_off(row, a, (128 / 8) * 128) | (j > 0 && key[j - 1] == k ? (uint32_t)CONT : 0u));
+        }
+        ofl[j] = flv[i];
+        oval[j] = val[i];
+        const int64_t s = seg_of(k), ps = j == 0 ? -1 : seg_of(key[j - 1]);
+        for (int64_t q = ps + 1; q <= s; ++q) seg_ptr[q] = (int32_t)j;
+        if (j == m - 1)
+            for (int64_t q = s + 1; q <= n_seg; ++q) seg_ptr[q] = (int32_t)m;
+    }
+}
+
+// Bits of the largest Σ|val| over the entries of one (atom, voxel) run of the DSC stream.
+template <class VT>
+__global__ void run_vmax_kernel(const uint16_t* __restrict__ soff, const VT* __restrict__ val, int64_t m,
+                                uint32_t* __restrict__ out) {
+    uint32_t best = 0u;
+    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
+        if (soff[j] & CONT) continue;
+        float sum = fabsf(load_val(val + j));
+        for (int64_t k = j + 1; k < m && (soff[k] & CONT); ++k) sum += fabsf(load_val(val + k));
+        best = max(best, __float_as_uint(sum));
+    }
+    for (int o = 16; o > 0; o >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, o));
+    if ((threadIdx.x & 31) == 0 && best) atomicMax(out, best);
 }
 
 template <class T>
@@ -728,9 +877,135 @@ static life_status assign_tiles(const life_index_s* ix, const std::vector<BrickS
     return LIFE_OK;
 }
 
+// The sorted form of the tables while the bricks are being formed: the entries by
+// (brick, fascicle), the heads of equal keys and their ranks.
+struct SortedTables {
+    TmpBuf slot, key, pay, head, uidx;
+    int32_t n_unique = 0;
+};
+
+static life_status sort_entries(const life_index_s* ix, const TileSet& H, const TmpBuf& slot, int order, int bits,
+                                TmpBuf& key, TmpBuf& pay, cudaStream_t s) {
+    const int64_t m = ix->nnz;
+    LIFE_TRY(key.alloc(sizeof(uint64_t) * m, s));
+    LIFE_TRY(pay.alloc(sizeof(uint32_t) * m, s));
+    entry_key_kernel<<<grid1d(m), 256, 0, s>>>(ix->vox.vox_ptr.as<int32_t>(), ix->nv, slot.as<int64_t>(),
+                                               H.tile_brick.as<int32_t>(), ix->vox.atom.as<uint16_t>(),
+                                               ix->vox.fasc.as<int32_t>(), m, order, ix->key_bits_f, key.as<uint64_t>(),
+                                               pay.as<uint32_t>());
+    LIFE_CHECK_LAUNCH();
+    return radix_sort_pairs(key, pay, m, 0, bits, s);
+}
+
+// Table offsets of the bricks (into L.brick_fasc_ptr) by sorting.
+static life_status sort_tables(life_index_s* ix, const TileSet& H, SortedTables& T, cudaStream_t s) {
+    const int64_t m = ix->nnz;
+    LIFE_TRY(T.slot.alloc(sizeof(int64_t) * ix->nv, s));
+    voxel_slot_kernel<<<grid1d(H.n_tiles * TILE_V), 256, 0, s>>>(H.tile_vox.as<int32_t>(), H.n_tiles * TILE_V,
+                                                                 T.slot.as<int64_t>());
+    LIFE_CHECK_LAUNCH();
+    LIFE_TRY(sort_entries(ix, H, T.slot, BY_TABLE, nbits64(H.n_bricks) + ix->key_bits_f, T.key, T.pay, s));
+    LIFE_TRY(T.head.alloc(sizeof(int32_t) * m, s));
+    LIFE_TRY(T.uidx.alloc(sizeof(int32_t) * m, s));
+    head_flag_kernel<<<grid1d(m), 256, 0, s>>>(T.key.as<uint64_t>(), m, T.head.as<int32_t>());
+    LIFE_CHECK_LAUNCH();
+    LIFE_TRY(exclusive_scan_i32(T.head.as<int32_t>(), T.uidx.as<int32_t>(), m, s));
+    int32_t last[2];
+    LIFE_CUDA_TRY(cudaMemcpyAsync(&last[0], T.uidx.as<int32_t>() + m - 1, 4, cudaMemcpyDeviceToHost, s));
+    LIFE_CUDA_TRY(cudaMemcpyAsync(&last[1], T.head.as<int32_t>() + m - 1, 4, cudaMemcpyDeviceToHost, s));
+    LIFE_CUDA_TRY(cudaStreamSynchronize(s));
+    T.n_unique = last[0] + last[1];
+    sorted_bptr_kernel<<<grid1d(m), 256, 0, s>>>(T.key.as<uint64_t>(), m, ix->key_bits_f, T.head.as<int32_t>(),
+                                                 T.uidx.as<int32_t>(), H.n_bricks, T.n_unique,
+                                                 ix->tile.brick_fasc_ptr.as<int32_t>());
+    LIFE_CHECK_LAUNCH();
+    return LIFE_OK;
+}
+
+// The rest of the sorted form: the tables and both streams.
+template <class VT>
+static life_status sort_tables_and_streams(life_index_s* ix, const TileSet& H, SortedTables& T, uint32_t* vmax,
+                                           cudaStream_t s) {
+    TileLayout& L = ix->tile;
+    const VT* val = ix->vox.val.as<VT>();
+    const int64_t m = ix->nnz;
+    const int bf = ix->key_bits_f, bt = nbits64(H.n_tiles), n_c = L.kp / DKC;
+    TmpBuf flv, first;
+    LIFE_TRY(flv.alloc(sizeof(uint16_t) * m, s));
+    LIFE_TRY(first.alloc(sizeof(int32_t) * T.n_unique, s));
+    sorted_table_kernel<<<grid1d(m), 256, 0, s>>>(T.key.as<uint64_t>(), T.pay.as<uint32_t>(), m, bf,
+                                                  T.head.as<int32_t>(), T.uidx.as<int32_t>(),
+                                                  L.brick_fasc_ptr.as<int32_t>(), L.brick_fasc.as<int32_t>(),
+                                                  first.as<int32_t>(), flv.as<uint16_t>());
+    LIFE_CHECK_LAUNCH();
+    if (L.wc_stream && sizeof(VT) == 2) {  // the FP32 WC sums in FP32 tables
+        TmpBuf mx;
+        LIFE_TRY(mx.alloc(2 * sizeof(uint32_t) * (size_t)H.n_bricks, s));
+        LIFE_CUDA_TRY(cudaMemsetAsync(mx.p, 0, 2 * sizeof(uint32_t) * (size_t)H.n_bricks, s));
+        uint32_t* cm = mx.as<uint32_t>();
+        sorted_cv_max_kernel<VT><<<grid1d(m), 256, 0, s>>>(T.key.as<uint64_t>(), T.pay.as<uint32_t>(), m, bf,
+                                                           T.head.as<int32_t>(), T.uidx.as<int32_t>(),
+                                                           first.as<int32_t>(), T.n_unique, val, cm, cm + H.n_bricks);
+        LIFE_CHECK_LAUNCH();
+        sorted_cv_kernel<<<grid1d(H.n_bricks), 256, 0, s>>>(cm, cm + H.n_bricks, H.n_bricks, L.brick_cv.as<float>());
+        LIFE_CHECK_LAUNCH();
+    }
+    for (TmpBuf* b : {&T.head, &T.uidx, &first}) b->release();
+    LIFE_TRY(sort_entries(ix, H, T.slot, BY_DSC, bt + 16, T.key, T.pay, s));
+    sorted_stream_kernel<VT, false><<<grid1d(m), 256, 0, s>>>(
+        T.key.as<uint64_t>(), T.pay.as<uint32_t>(), m, flv.as<uint16_t>(), val, n_c, L.n_sub, 0, H.n_tiles * n_c,
+        L.soff.as<uint16_t>(), L.fl.as<uint16_t>(), L.val.as<VT>(), L.chunk_ptr.as<int32_t>());
+    LIFE_CHECK_LAUNCH();
+    run_vmax_kernel<VT><<<grid1d(m), 256, 0, s>>>(L.soff.as<uint16_t>(), L.val.as<VT>(), m, vmax);
+    LIFE_CHECK_LAUNCH();
+    if (!L.wc_stream) return LIFE_OK;
+    LIFE_TRY(sort_entries(ix, H, T.slot, BY_WC, bt + 16, T.key, T.pay, s));
+    sorted_stream_kernel<VT, true><<<grid1d(m), 256, 0, s>>>(
+        T.key.as<uint64_t>(), T.pay.as<uint32_t>(), m, flv.as<uint16_t>(), val, n_c, L.n_sub, sizeof(VT) == 4 ? 1 : 0,
+        H.n_tiles * 4 * L.n_sub, L.wkey.as<uint16_t>(), L.wfl.as<uint16_t>(), L.wval.as<VT>(),
+        L.wseg_ptr.as<int32_t>());
+    LIFE_CHECK_LAUNCH();
+    return LIFE_OK;
+}
+
+// Whether the layout is sooner there by sorting than by counting, from the entries of
+// each tile (base) and of its fullest quarter of 32 rows, in microseconds fitted to builds
+// timed both ways on one GB300.  Counting: a stream pass 9 us and 0.5 ns an entry walked,
+// the first walk and one more for every TS_STAGE entries of the pass; a window of a brick's
+// table 9 us, and three walks at 0.8 ns an entry, or 12 ns where one warp's 32 rows hold
+// most of them; the fullest brick and tile, or the SMs' even share if that is more.
+// Sorting: 0.5 ms and 0.25 ns an entry, wherever the entries lie.  Whole builds, BF16,
+// counted / sorted: 80M entries in 500k voxels 15.7 / 30.0 ms, 10M in 32768 voxels 3.5 /
+// 5.3; 3M in 4096 2.9 / 2.9, 6M there 4.6 / 3.8; 1M in 128 25 / 1.8, 10M in 128 1515 /
+// 4.8; 50M in 4M voxels with 5M fascicles 29.7 / 22.0, with 50M fascicles 120 / 23.
+static bool sort_is_faster(const std::vector<int32_t>& base, const std::vector<int32_t>& quarter,
+                           const std::vector<int32_t>& btile, int n_c, bool wc, int64_t nf, int window, int num_sms) {
+    constexpr double PASS = 9.0, WALK = 5.0e-4, WINDOW = 9.0, TABLE_WALK = 8.0e-4, ROWS_WALK = 0.012, SORT = 500.0,
+                     SORT_ENTRY = 2.5e-4;
+    const double sms = std::max(num_sms, 1), windows = (double)((nf + window - 1) / window);
+    double tab = 0.0, tab_max = 0.0, str = 0.0, str_max = 0.0;
+    for (size_t b = 0; b + 1 < btile.size(); ++b) {
+        double most = 0.0;
+        for (int32_t t = btile[b]; t < btile[b + 1]; ++t) {
+            const double e = base[t + 1] - base[t], q = quarter[t];
+            double us = PASS * n_c + WALK * e * (2.0 + e / n_c / TS_STAGE);
+            if (wc) us += PASS * 4 + WALK * e * (2.0 + q / TS_STAGE);
+            str += us;
+            str_max = std::max(str_max, us);
+            most = std::max(most, q);
+        }
+        const double e = base[btile[b + 1]] - base[btile[b]];
+        const double us = windows * (WINDOW + 3.0 * std::max(ROWS_WALK * most, TABLE_WALK * e));
+        tab += us;
+        tab_max = std::max(tab_max, us);
+    }
+    return std::max(tab_max, tab / sms) + std::max(str_max, str / sms) > SORT + SORT_ENTRY * base.back();
+}
+
 template <class VT>
 static life_status build_tables_and_streams(life_index_s* ix, const TileSet& H, const int32_t* tile_base, int window,
-                                            uint32_t* vmax, cudaStream_t s) {
+                                            SortedTables* sorted, uint32_t* vmax, cudaStream_t s) {
+    if (sorted) return sort_tables_and_streams<VT>(ix, H, *sorted, vmax, s);
     TileLayout& L = ix->tile;
     const VoxelLayout& V = ix->vox;
     const int64_t m = ix->nnz;
@@ -889,9 +1164,10 @@ life_status build_tile_layout(life_index_s* ix, cudaStream_t s) {
     L.n_sub = L.kp / SUB;
     const int bf = ix->key_bits_f;
     TileSet H;
-    std::vector<int32_t> hbptr, hgroup;
-    TmpBuf count;
-    bool ok = false;
+    SortedTables ST;
+    std::vector<int32_t> hbptr, hgroup, hbase, hquarter, hbtile;
+    TmpBuf count, tcount, tquarter, tbase;
+    bool ok = false, sorted = false;
     const int window = bt_window(ix->nf);
     const size_t csm = (size_t)window / 8;
     LIFE_CUDA_TRY(cudaFuncSetAttribute(brick_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm));
@@ -909,14 +1185,32 @@ life_status build_tile_layout(life_index_s* ix, cudaStream_t s) {
             set_error("tensor-core layout: sort key too wide");
             return LIFE_ENOTSUP;
         }
-        LIFE_TRY(count.alloc(sizeof(int32_t) * ((size_t)H.n_bricks + 1), s));
+        LIFE_TRY(tcount.alloc(sizeof(int32_t) * (H.n_tiles + 1), s));
+        LIFE_TRY(tquarter.alloc(sizeof(int32_t) * (H.n_tiles + 1), s));
+        LIFE_TRY(tbase.alloc(sizeof(int32_t) * (H.n_tiles + 1), s));
+        tile_count_kernel<<<(unsigned)((H.n_tiles + 8) / 8), 256, 0, s>>>(
+            H.tile_vox.as<int32_t>(), ix->vox.vox_ptr.as<int32_t>(), H.n_tiles, tcount.as<int32_t>(),
+            tquarter.as<int32_t>());
+        LIFE_CHECK_LAUNCH();
+        LIFE_TRY(exclusive_scan_i32(tcount.as<int32_t>(), tbase.as<int32_t>(), H.n_tiles + 1, s));
+        LIFE_TRY(download(hbase, tbase.p, (size_t)H.n_tiles + 1, s));
+        LIFE_TRY(download(hquarter, tquarter.p, (size_t)H.n_tiles, s));
+        LIFE_TRY(download(hbtile, H.brick_tile_ptr.p, (size_t)H.n_bricks + 1, s));
+        LIFE_CUDA_TRY(cudaStreamSynchronize(s));
+        sorted = m > 0 && sort_is_faster(hbase, hquarter, hbtile, L.kp / DKC, L.wc_stream, ix->nf, window, ix->num_sms);
         L.brick_fasc_ptr.release();
         LIFE_TRY(L.brick_fasc_ptr.alloc(sizeof(int32_t) * ((size_t)H.n_bricks + 1)));
-        brick_count_kernel<<<(unsigned)std::min<int64_t>(H.n_bricks, 65535), BT_THREADS, csm, s>>>(
-            H.tile_vox.as<int32_t>(), ix->vox.vox_ptr.as<int32_t>(), ix->vox.fasc.as<int32_t>(),
-            H.brick_tile_ptr.as<int32_t>(), H.n_bricks, ix->nf, window, count.as<int32_t>());
-        LIFE_CHECK_LAUNCH();
-        LIFE_TRY(exclusive_scan_i32(count.as<int32_t>(), L.brick_fasc_ptr.as<int32_t>(), (int64_t)H.n_bricks + 1, s));
+        if (sorted) {
+            LIFE_TRY(sort_tables(ix, H, ST, s));
+        } else {
+            LIFE_TRY(count.alloc(sizeof(int32_t) * ((size_t)H.n_bricks + 1), s));
+            brick_count_kernel<<<(unsigned)std::min<int64_t>(H.n_bricks, 65535), BT_THREADS, csm, s>>>(
+                H.tile_vox.as<int32_t>(), ix->vox.vox_ptr.as<int32_t>(), ix->vox.fasc.as<int32_t>(),
+                H.brick_tile_ptr.as<int32_t>(), H.n_bricks, ix->nf, window, count.as<int32_t>());
+            LIFE_CHECK_LAUNCH();
+            LIFE_TRY(exclusive_scan_i32(count.as<int32_t>(), L.brick_fasc_ptr.as<int32_t>(), (int64_t)H.n_bricks + 1,
+                                        s));
+        }
         LIFE_TRY(download(hbptr, L.brick_fasc_ptr.p, (size_t)H.n_bricks + 1, s));
         if (grouped) LIFE_TRY(download(hgroup, H.brick_group.p, (size_t)H.n_bricks, s));
         LIFE_CUDA_TRY(cudaStreamSynchronize(s));
@@ -984,19 +1278,14 @@ life_status build_tile_layout(life_index_s* ix, cudaStream_t s) {
     }
     LIFE_TRY(L.brick_cv.alloc(sizeof(float) * std::max<int64_t>(H.n_bricks, 1)));
     LIFE_TRY(L.tile_amax.alloc(sizeof(uint32_t) * 4 * std::max<int64_t>(H.n_tiles, 1)));
-    TmpBuf tcount, tbase, rv;
-    LIFE_TRY(tcount.alloc(sizeof(int32_t) * (H.n_tiles + 1), s));
-    LIFE_TRY(tbase.alloc(sizeof(int32_t) * (H.n_tiles + 1), s));
+    TmpBuf rv;
     LIFE_TRY(rv.alloc(sizeof(uint32_t), s));
     LIFE_CUDA_TRY(cudaMemsetAsync(rv.p, 0, sizeof(uint32_t), s));
-    tile_count_kernel<<<(unsigned)((H.n_tiles + 8) / 8), 256, 0, s>>>(
-        H.tile_vox.as<int32_t>(), ix->vox.vox_ptr.as<int32_t>(), H.n_tiles, tcount.as<int32_t>());
-    LIFE_CHECK_LAUNCH();
-    LIFE_TRY(exclusive_scan_i32(tcount.as<int32_t>(), tbase.as<int32_t>(), H.n_tiles + 1, s));
+    SortedTables* st = sorted ? &ST : nullptr;
     if (L.vbytes == 4)
-        LIFE_TRY(build_tables_and_streams<float>(ix, H, tbase.as<int32_t>(), window, rv.as<uint32_t>(), s));
+        LIFE_TRY(build_tables_and_streams<float>(ix, H, tbase.as<int32_t>(), window, st, rv.as<uint32_t>(), s));
     else
-        LIFE_TRY(build_tables_and_streams<__nv_bfloat16>(ix, H, tbase.as<int32_t>(), window, rv.as<uint32_t>(), s));
+        LIFE_TRY(build_tables_and_streams<__nv_bfloat16>(ix, H, tbase.as<int32_t>(), window, st, rv.as<uint32_t>(), s));
     std::vector<int32_t> wptr(H.n_bricks + 1, 0);
     {
         // padded, 16-byte aligned per-brick weight slots for the DSC's bulk table loads
@@ -1046,10 +1335,7 @@ life_status build_tile_layout(life_index_s* ix, cudaStream_t s) {
         L.tile_brick.release();
     }
     // largest bricks first
-    std::vector<int32_t> hbase, hbtile;
     uint32_t vbits = 0u;
-    LIFE_TRY(download(hbase, tbase.p, (size_t)H.n_tiles + 1, s));
-    LIFE_TRY(download(hbtile, H.brick_tile_ptr.p, (size_t)H.n_bricks + 1, s));
     LIFE_CUDA_TRY(cudaMemcpyAsync(&vbits, rv.p, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     LIFE_CUDA_TRY(cudaStreamSynchronize(s));
     std::memcpy(&L.run_vmax, &vbits, sizeof(float));
