@@ -1226,12 +1226,21 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
                                              max(abs_bits(yv.z), abs_bits(yv.w)));
                                 }
                             } else {
-                                for (int k = 0; k < nth; ++k) {
-                                    float y = trow[k] * y_unscale;
-                                    if (A.b) y -= __ldg(A.b + o + k);
-                                    if (wy) A.out[o + k] = y;
-                                    sqf += y * y;
-                                    am = max(am, abs_bits(y));
+                                // (eight b values on their way at a time, not each waited for:
+                                // 64000 voxels of 15 entries, Nθ = 33: 107 -> 55 us a DSC with b)
+                                for (int k0 = 0; k0 < nth; k0 += 8) {
+                                    float bk[8];
+#pragma unroll
+                                    for (int e = 0; e < 8; ++e)
+                                        bk[e] = (A.b && k0 + e < nth) ? __ldg(A.b + o + k0 + e) : 0.0f;
+#pragma unroll
+                                    for (int e = 0; e < 8; ++e) {
+                                        if (k0 + e >= nth) break;
+                                        const float y = trow[k0 + e] * y_unscale - bk[e];
+                                        if (wy) A.out[o + k0 + e] = y;
+                                        sqf += y * y;
+                                        am = max(am, abs_bits(y));
+                                    }
                                 }
                             }
                         }
