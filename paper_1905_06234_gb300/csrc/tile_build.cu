@@ -22,6 +22,7 @@
 #include <numeric>
 #include <vector>
 
+#include "launch_rules.cuh"
 #include "tile_layout.cuh"
 #include "tc_ptx.cuh"
 
@@ -1047,92 +1048,6 @@ static life_status build_tables_and_streams(life_index_s* ix, const TileSet& H, 
     return LIFE_OK;
 }
 
-// Shares the tiles out to the CTAs of a launch (at most one per SM), as units of one
-// brick's consecutive tiles; each unit pays for its brick's fascicle table (gathered
-// by the DSC, flushed by the WC).  Two ways:
-//  - whole bricks, largest first, dealt to the CTAs in snake order: at the paper's size
-//    (6 bricks a CTA) the CTAs' times are within 3 % of one another;
-//  - the tiles in brick order, cut into one run per CTA of about equal cost, wherever
-//    in a brick the cut falls, at the price of the cut bricks' tables twice.  Whole
-//    bricks leave most SMs without any on the 16^3 workload (8 bricks of 4 tiles: a
-//    DSC took 47 us, 25 with the tiles dealt out) and give the CTAs of the 64^3 one
-//    three or four (512 bricks on 152 SMs: 142 -> 130 us).
-// The one whose most loaded CTA has less to do is taken (whole bricks unless the other
-// is better by 5 %).  The costs, in units of an entry's time, are those of the BF16
-// kernels' phases on the 64^3 and the paper workload: a tile 7 us, a table slot 0.8 ns,
-// a unit 2 us, an entry 0.14 ns.  A batch, whose problems stop at different times,
-// always deals: bricks, or single tiles when they are fewer than two per SM.
-struct WorkShare {
-    std::vector<int32_t> brick, t0, t1, cta_unit{0};
-    double worst = 0.0;
-    int grid() const { return (int)cta_unit.size() - 1; }
-};
-
-static WorkShare share_out(const std::vector<int32_t>& order, const std::vector<int32_t>& btile,
-                           const std::vector<int32_t>& base, const std::vector<int32_t>& bfasc, int num_sms,
-                           bool batch) {
-    constexpr double TILE_COST = 50000.0, UNIT_COST = 14000.0, SLOT_COST = 6.0;
-    const int nb = (int)btile.size() - 1, nt = btile[nb], sms = std::max(num_sms, 1);
-    auto unit_cost = [&](int b) { return UNIT_COST + SLOT_COST * (bfasc[b + 1] - bfasc[b]); };
-    auto tile_cost = [&](int t) { return TILE_COST + (base[t + 1] - base[t]); };
-    auto add = [](WorkShare& W, int b, int t0, int t1) {
-        W.brick.push_back(b);
-        W.t0.push_back(t0);
-        W.t1.push_back(t1);
-    };
-    WorkShare deal;
-    if (batch && nb < 2 * sms) {
-        std::vector<int32_t> tbrick(nt);
-        for (int b = 0; b < nb; ++b)
-            for (int t = btile[b]; t < btile[b + 1]; ++t) tbrick[t] = b;
-        const int grid = std::min(sms, nt);
-        for (int c = 0; c < grid; ++c) {
-            for (int t = c; t < nt; t += grid) add(deal, tbrick[t], t, t + 1);
-            deal.cta_unit.push_back((int32_t)deal.brick.size());
-        }
-        return deal;
-    }
-    const int dgrid = std::min(sms, nb);
-    for (int c = 0; c < dgrid; ++c) {
-        double cost = 0.0;
-        for (int r = 0;; ++r) {
-            const int k = r * dgrid + ((r & 1) ? (dgrid - 1 - c) : c);
-            if (k >= nb) break;
-            const int b = order[k];
-            add(deal, b, btile[b], btile[b + 1]);
-            cost += unit_cost(b);
-            for (int t = btile[b]; t < btile[b + 1]; ++t) cost += tile_cost(t);
-        }
-        deal.cta_unit.push_back((int32_t)deal.brick.size());
-        deal.worst = std::max(deal.worst, cost);
-    }
-    if (batch) return deal;
-    WorkShare cut;
-    double left = 0.0;
-    for (int b = 0; b < nb; ++b) left += unit_cost(b);
-    for (int t = 0; t < nt; ++t) left += tile_cost(t);
-    const int grid = std::min(sms, nt);
-    for (int c = 0, b = 0, t = 0; c < grid; ++c) {
-        const double want = left / (grid - c);
-        double cost = 0.0;
-        const int more = grid - 1 - c;  // each CTA after this one takes a tile at least
-        while (t < nt - more) {
-            const bool opens = cost == 0.0 || t == btile[b];
-            const double x = tile_cost(t) + (opens ? unit_cost(b) : 0.0);
-            if (more > 0 && cost > 0.0 && cost + 0.5 * x > want) break;
-            if (opens) add(cut, b, t, t);
-            cut.t1.back() = ++t;
-            cost += x;
-            if (t == btile[b + 1]) ++b;
-        }
-        left -= cost;
-        if (t < nt && t != btile[b]) left += unit_cost(b);  // a cut brick's table is paid for again
-        cut.cta_unit.push_back((int32_t)cut.brick.size());
-        cut.worst = std::max(cut.worst, cost);
-    }
-    return cut.worst < 0.95 * deal.worst ? cut : deal;
-}
-
 life_status build_tile_layout(life_index_s* ix, cudaStream_t s) {
     TileLayout& L = ix->tile;
     if (ix->na > 512 || ix->nt > 128) {
@@ -1346,7 +1261,7 @@ life_status build_tile_layout(life_index_s* ix, cudaStream_t s) {
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return bnnz[x] > bnnz[y]; });
     LIFE_TRY(upload(L.brick_order, order, s));
-    const WorkShare W = share_out(order, hbtile, hbase, hbptr, ix->num_sms, grouped);
+    const WorkShare W = share_out(order, hbtile, hbase, hbptr, ix->num_sms, grouped, L.vbytes == 4);
     L.grid = W.grid();
     L.n_units = (int32_t)W.brick.size();
     std::vector<int32_t> units = W.cta_unit;
