@@ -104,4 +104,39 @@ inline WorkShare share_out(const std::vector<int32_t>& order, const std::vector<
     return other.worst < line * deal.worst ? other : deal;
 }
 
+// Form of a BF16 DSC launch.  y_tile: b and Y pass through a tile in shared memory (where
+// it fits beside the brick table and two S stages, and rows are 16-byte aligned: can);
+// stages: S stages.  The lines, from DSC calls timed in each form (us, one GB300; entries
+// per tile and 128-atom chunk):
+//  - The tile of Y saves the epilogue's reads of b, which a tile of several chunks hides
+//    behind nothing (64^3 voxels, Nθ 96, Na 360: 339 entries 128 -> 106, 3812 177 -> 146,
+//    and 40^3 at 7621 the same either way).  A tile of one chunk is over before its b has
+//    arrived (Nθ 64, Na 128: 1005 81 -> 87, 7536 106 -> 109, 16351 132 -> 123, 22635 160 ->
+//    140): it takes the tile from 16384 entries on.  Bricks of one tile gather a table for
+//    every tile, and there the copies only delay (4^3 bricks, 48^3 voxels: 1270 112 -> 104,
+//    2752 126 -> 129, 4978 147 -> 167): up to 2304.
+//  - A third and fourth stage let idle producers start on the next chunks: worth it where
+//    a chunk's 256-entry blocks are for at most half of the 23 producer warps and a tile has
+//    more than two chunks (64^3, Nθ 32, Na 512: 255 105 -> 81, 2864 137 -> 135, 7481 208 ->
+//    226; Nθ 64, Na 360: 339 99 -> 97, 3812 130 -> 134, 5510 150 -> 158; Na 181: 1893 83 ->
+//    89, 7422 120 -> 155).
+constexpr int DSTAGE = 2;      // S stages of the general form, and the
+constexpr int DSTAGE_MAX = 4;  // most the form with the tile of Y takes
+
+struct DscForm {
+    bool y_tile = false;
+    int stages = DSTAGE;
+};
+
+template <class Fits>  // fits(stages): the form with the tile of Y and so many stages fits shared memory
+inline DscForm dsc_form(int64_t n_nnz, int64_t n_tiles, int64_t n_bricks, int n_c, bool can, Fits fits) {
+    DscForm F;
+    const int64_t chunks = n_tiles * n_c;
+    const bool pays = n_c == 1 ? n_nnz >= 16384 * chunks : n_tiles >= 2 * n_bricks || n_nnz <= 2304 * chunks;
+    F.y_tile = can && pays && fits(DSTAGE);
+    if (F.y_tile && n_c > 2 && n_nnz <= 23 * 256 / 2 * chunks)
+        while (F.stages < DSTAGE_MAX && fits(F.stages + 1)) ++F.stages;
+    return F;
+}
+
 }  // namespace life

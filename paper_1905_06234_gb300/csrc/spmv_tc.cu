@@ -18,6 +18,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "launch_rules.cuh"
 #include "tile_layout.cuh"
 #include "tc_ptx.cuh"
 
@@ -525,8 +526,6 @@ constexpr int DSC_EPI_WARPS = 4;
 constexpr int DSC_MMA_WARP = DSC_PROD_WARPS + DSC_EPI_WARPS;
 constexpr int DSC_THREADS = (DSC_MMA_WARP + 1) * 32;
 constexpr int DSC_PROD_THREADS = DSC_PROD_WARPS * 32;
-constexpr int DSTAGE = 2;                                 // S-chunk ring depth, and the deepest the
-constexpr int DSTAGE_MAX = 4;                             // small-table form takes
 constexpr uint32_t DS_BYTES = TILE_V * DKC * 2;           // one S chunk: 128 rows x 128 atoms, bf16
 constexpr uint32_t DS_SBO = (DKC / 8) * 128;              // 8-row group stride of an S chunk
 
@@ -820,11 +819,10 @@ __global__ void __launch_bounds__(PREP_THREADS) tc_prep_kernel(PrepArgs P) {
 //  - up to four S stages as they fit, and the warp that takes a chunk's first block
 //    moves on by DSC_ROT from chunk to chunk (the same three of the 23 producers had
 //    all the work).
-// 64^3 workload: 130 -> 108 us with b, an iteration 418 -> 367 us.  It is
-// taken where the tile of Y fits beside two stages: with tables of the paper's size it
-// does not, and there the tiles are dense, the producers bound the kernel, and a third
-// stage alone only costs (one-third paper workload 112 -> 127 us).  FP32 storage, whose
-// accumulator has θ along the lanes, lost by it (64^3: 176 -> 306 us).
+// 64^3 workload: 130 -> 108 us with b, an iteration 418 -> 367 us.  Where it is taken, and
+// with how many stages, is dsc_form's rule (with tables of the paper's size it does not
+// fit).  FP32 storage, whose accumulator has θ along the lanes, lost by it (64^3: 176 ->
+// 306 us).
 constexpr int DSC_ROT = 7;
 
 template <bool F32, bool SMALL>
@@ -2478,16 +2476,13 @@ life_status dsc_tc(life_index_s* ix, const float* D, const float* w, const float
         A.val = nullptr;
         A.val32 = L.val.as<float>();
     }
-    // the small-table form where a tile of Y fits beside the table, with as many S stages
-    // as fit then
     int optin = 0;
     LIFE_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ix->device));
-    auto fits = [&](int stages, bool y_tile) {
-        return dsc_smem_bytes(A.np, A.kp, A.nt, A.max_fb, f32, stages, y_tile) + 512 <= (uint32_t)optin;
-    };
-    A.y_tile = !f32 && A.vec4 && fits(DSTAGE, true) ? 1 : 0;
-    A.dstage = DSTAGE;
-    while (A.y_tile && A.dstage < DSTAGE_MAX && fits(A.dstage + 1, true)) ++A.dstage;
+    const DscForm form = dsc_form(L.n_nnz, L.n_tiles, L.n_bricks, A.kp / DKC, !f32 && A.vec4, [&](int stages) {
+        return dsc_smem_bytes(A.np, A.kp, A.nt, A.max_fb, f32, stages, true) + 512 <= (uint32_t)optin;
+    });
+    A.y_tile = form.y_tile ? 1 : 0;
+    A.dstage = form.stages;
     const uint32_t smem = dsc_smem_bytes(A.np, A.kp, A.nt, A.max_fb, f32, A.dstage, A.y_tile != 0);
     const bool sparse = L.sparse && !bg.live && L.wb_total > 0 && L.n_nnz > 0;
     if (sparse) {

@@ -1,5 +1,5 @@
 """The host-side rules that shape the tensor-core launches, compiled here with the host
-compiler: how a launch's tiles are shared out to the CTAs."""
+compiler: how a launch's tiles are shared out to the CTAs, and the form of a BF16 DSC."""
 import ctypes
 import os
 import shutil
@@ -21,6 +21,10 @@ extern "C" int share(const int* order, const int* btile, const int* base, const 
     std::copy(W.t0.begin(), W.t0.end(), t0);
     std::copy(W.t1.begin(), W.t1.end(), t1);
     return W.grid();
+}
+extern "C" int form(long long nnz, long long tiles, long long bricks, int n_c, int can, int max_stages) {
+    const auto F = life::dsc_form(nnz, tiles, bricks, n_c, can != 0, [&](int stages) { return stages <= max_stages; });
+    return F.y_tile ? F.stages : -F.stages;
 }
 """
 
@@ -91,3 +95,20 @@ def test_share(rules, nb, entries, slots, spread, batch, fp32):
         assert (seen == 1).all()
         # never a worse share than whole bricks (10 % in the batches of FP32 storage, which measure better)
         assert makespan(lay, cta_unit, (brick, t0, t1)) <= (1.1 if batch and fp32 else 1.0) * whole_bricks(lay, sms)
+
+
+# the form measured fastest (4, 3, 2: with the tile of Y and so many stages; -2: general), by entries
+# per tile and chunk, chunks a tile, tiles a brick, stages that fit
+@pytest.mark.parametrize("epc,n_c,per_brick,fit,best", [
+    (339, 3, 4, 3, 3), (3812, 3, 4, 3, 2), (7621, 3, 4, 2, 2), (255, 4, 4, 4, 4), (2864, 4, 4, 4, 4), (7481, 4, 4, 4, 2),
+    (1005, 1, 4, 4, -2), (7536, 1, 4, 4, -2), (22635, 1, 4, 4, 2), (29545, 1, 4, 4, 2), (1893, 2, 4, 4, 2),
+    (12525, 2, 2, 4, 2), (1270, 3, 1, 2, 2), (4756, 3, 1, 2, -2), (8603, 3, 1, 2, -2), (339, 3, 4, 1, -2)])
+def test_dsc_form(rules, epc, n_c, per_brick, fit, best):
+    tiles = 1000 * per_brick
+    args = lambda can: [ctypes.c_longlong(x) for x in (epc * tiles * n_c, tiles, 1000)] + [n_c, can, fit]
+    assert rules.form(*args(1)) == best
+    assert rules.form(*args(0)) == -2       # FP32 storage, or rows off a 16-byte boundary
+
+
+def test_dsc_form_of_an_empty_index(rules):
+    assert rules.form(ctypes.c_longlong(0), ctypes.c_longlong(1), ctypes.c_longlong(1), 1, 1, 4) == -2
