@@ -502,12 +502,10 @@ life_status build_voxel_layout(life_index_s* ix, const int32_t* atom, const int3
 
 // ------------------------------------------------------------ re-sorting
 
-// Voxel of each entry of the merged list (one warp per voxel).
-__global__ void entry_voxel_kernel(const int32_t* __restrict__ vox_ptr, int32_t nv, int32_t* __restrict__ voxel) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t v = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; v < nv; v += warps)
-        for (int32_t i = vox_ptr[v] + lane; i < vox_ptr[v + 1]; i += 32) voxel[i] = (int32_t)v;
+// Voxel of each entry of the merged list.
+__global__ void entry_voxel_kernel(const int32_t* __restrict__ vox_ptr, int32_t nv, int64_t m,
+                                   int32_t* __restrict__ voxel) {
+    for_entry_segments(vox_ptr, nv, m, [&](int64_t i, int64_t v) { voxel[i] = (int32_t)v; });
 }
 
 // Re-keys the merged (v, a, f) list in another order; payload = merged position.
@@ -561,16 +559,21 @@ life_status export_layout(life_index_s* ix, int layout, int32_t* atom, int32_t* 
     }
     const int64_t m = ix->nnz;
     if (m == 0) return LIFE_OK;
+    // the voxel of each entry: straight into the output in the list's own order, else
+    // through a temporary that the permutation reads
+    const bool own = layout == LIFE_LAYOUT_VOXEL;
     TmpBuf vox, perm;
-    LIFE_TRY(vox.alloc(sizeof(int32_t) * m, s));
-    entry_voxel_kernel<<<grid_for((int64_t)ix->nv * 32), 256, 0, s>>>(ix->vox.vox_ptr.as<int32_t>(), ix->nv,
-                                                                      vox.as<int32_t>());
-    LIFE_CHECK_LAUNCH();
+    if (!own) LIFE_TRY(vox.alloc(sizeof(int32_t) * m, s));
+    int32_t* vdst = own ? voxel : vox.as<int32_t>();
+    if (vdst) {
+        entry_voxel_kernel<<<entry_segments_grid(m), 256, 0, s>>>(ix->vox.vox_ptr.as<int32_t>(), ix->nv, m, vdst);
+        LIFE_CHECK_LAUNCH();
+    }
     LIFE_TRY(layout_perm(ix, layout, vox.as<int32_t>(), perm, s));
     const float* x = ix->precision == LIFE_BF16 ? ix->uval.as<float>() : ix->vox.val.as<float>();
     gather_export_kernel<<<grid_for(m), 256, 0, s>>>(vox.as<int32_t>(), ix->vox.atom.as<uint16_t>(),
                                                      ix->vox.fasc.as<int32_t>(), x, perm.as<uint32_t>(), m, atom,
-                                                     voxel, fasc, val);
+                                                     own ? nullptr : voxel, fasc, val);
     LIFE_CHECK_LAUNCH();
     LIFE_CUDA_TRY(cudaStreamSynchronize(s));
     return LIFE_OK;

@@ -386,6 +386,68 @@ __device__ __forceinline__ bool gate_skip(const life_sbb_state* st, int mode) {
     return false;
 }
 
+// Last s in [lo, hi] with ptr[s] <= x (ptr ascending, ptr[lo] <= x), searched by the 32
+// lanes of a warp together.
+__device__ __forceinline__ int64_t warp_last_le(const int32_t* __restrict__ ptr, int64_t lo, int64_t hi, int64_t x) {
+    while (lo < hi) {
+        const int64_t step = (hi - lo) / 32 + 1, p = lo + step * ((threadIdx.x & 31) + 1);
+        const uint32_t le = __ballot_sync(0xffffffffu, p <= hi && __ldg(ptr + p) <= x);
+        lo += step * __popc(le);
+        hi = min(hi, lo + step - 1);
+    }
+    return lo;
+}
+
+// Calls f(i, s) for every entry i < m and the segment s of ptr [n_seg + 1] it lies in.  Each
+// warp of a launch of entry_segments_grid(m) blocks of 256 takes an equal run of entries,
+// whose few segments it finds once; neither long segments nor many empty ones hold up a warp.
+template <class F>
+__device__ __forceinline__ void for_entry_segments(const int32_t* __restrict__ ptr, int64_t n_seg, int64_t m, F f) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5, warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t per = (m + 128 * warps - 1) / (128 * warps) * 128, b = warp * per, e = min(b + per, m);
+    if (b >= e) return;
+    const int64_t last = warp_last_le(ptr, 0, n_seg - 1, e - 1);
+    int64_t cur = warp_last_le(ptr, 0, last, b);  // segment of the step's first entry, or of the one before it
+    constexpr int U = 4;                          // entries a lane and step
+    for (int64_t i0 = b; i0 < e; i0 += 32 * U) {
+        int64_t s[U];
+        // the starts of the 32 segments after cur: those inside this step are few
+        const int32_t p = cur + 1 + lane <= last ? __ldg(ptr + cur + 1 + lane) : INT32_MAX;
+        const int n = __popc(__ballot_sync(0xffffffffu, p <= i0 + 32 * U - 1));
+        if (n < 32) {
+            int c[U] = {};
+            for (int k = 0; k < n; ++k) {
+                const int32_t q = __shfl_sync(0xffffffffu, p, k) - (int32_t)i0;
+#pragma unroll
+                for (int u = 0; u < U; ++u) c[u] += q <= 32 * u + lane ? 1 : 0;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) s[u] = cur + c[u];
+        } else {  // many empty or short ones: each entry is searched for by itself
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                int64_t hi = last;
+                s[u] = cur;
+                while (s[u] < hi) {
+                    const int64_t mid = (s[u] + hi + 1) >> 1;
+                    if (__ldg(ptr + mid) <= i0 + 32 * u + lane) s[u] = mid;
+                    else hi = mid - 1;
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i0 + 32 * u + lane < e) f(i0 + 32 * u + lane, s[u]);
+        cur = __shfl_sync(0xffffffffu, s[U - 1], 31);
+    }
+}
+
 int device_sm_count();
+
+inline unsigned entry_segments_grid(int64_t m) {
+    const int64_t b = (m + 255) / 256, cap = (int64_t)device_sm_count() * 8;
+    return (unsigned)(b < 1 ? 1 : b < cap ? b : cap);
+}
 
 }  // namespace life

@@ -297,17 +297,11 @@ __global__ void export_fl_kernel(const uint16_t* __restrict__ fl, const uint16_t
 // 128-atom chunk from the entry's place in chunk_ptr (n_seg chunks, n_c per tile).
 __global__ void export_va_kernel(const uint16_t* __restrict__ soff, const int32_t* __restrict__ chunk_ptr,
                                  int64_t n_seg, int n_c, int64_t n, uint16_t* __restrict__ out) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t lo = 0, hi = n_seg - 1;  // the last chunk that starts at or before i
-        while (lo < hi) {
-            const int64_t mid = (lo + hi + 1) >> 1;
-            if (chunk_ptr[mid] <= i) lo = mid;
-            else hi = mid - 1;
-        }
+    for_entry_segments(chunk_ptr, n_seg, n, [&](int64_t i, int64_t s) {
         const uint32_t so = soff[i] & 0x7FFFu;
         const uint32_t row = (so >> 11) * 8 + ((so >> 4) & 7u), a = ((so >> 7) & 15u) * 8 + ((so >> 1) & 7u);
-        out[i] = (uint16_t)(row | ((a + (uint32_t)(lo % n_c) * DKC) << 7));
-    }
+        out[i] = (uint16_t)(row | ((a + (uint32_t)s % (uint32_t)n_c * DKC) << 7));
+    });
 }
 
 life_status export_tiles(life_index_s* ix, int32_t* tile_vox, int32_t* chunk_ptr, int32_t* brick_tile_ptr,
@@ -325,8 +319,8 @@ life_status export_tiles(life_index_s* ix, int32_t* tile_vox, int32_t* chunk_ptr
     LIFE_TRY(cp(brick_fasc, L.brick_fasc, L.brick_fasc.bytes));
     LIFE_TRY(cp(brick_order, L.brick_order, sizeof(int32_t) * L.n_bricks));
     if (va && L.n_nnz > 0) {
-        export_va_kernel<<<grid1d(L.n_nnz), 256, 0, s>>>(L.soff.as<uint16_t>(), L.chunk_ptr.as<int32_t>(),
-                                                         L.n_tiles * (L.kp / DKC), L.kp / DKC, L.n_nnz, va);
+        export_va_kernel<<<entry_segments_grid(L.n_nnz), 256, 0, s>>>(L.soff.as<uint16_t>(), L.chunk_ptr.as<int32_t>(),
+                                                              L.n_tiles * (L.kp / DKC), L.kp / DKC, L.n_nnz, va);
         LIFE_CHECK_LAUNCH();
     }
     if (fl && L.n_nnz > 0) {

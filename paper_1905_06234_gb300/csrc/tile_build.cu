@@ -658,20 +658,14 @@ __global__ void entry_key_kernel(const int32_t* __restrict__ vox_ptr, int32_t nv
                                  const int32_t* __restrict__ tile_brick, const uint16_t* __restrict__ atom,
                                  const int32_t* __restrict__ fasc, int64_t m, int order, int bf,
                                  uint64_t* __restrict__ key, uint32_t* __restrict__ payload) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-        int32_t lo = 0, hi = nv - 1;  // the entry's voxel: the last that starts at or before it
-        while (lo < hi) {
-            const int32_t mid = lo + (hi - lo + 1) / 2;
-            if (__ldg(vox_ptr + mid) <= i) lo = mid;
-            else hi = mid - 1;
-        }
-        const int64_t s = slot[lo], t = s / TILE_V;
+    for_entry_segments(vox_ptr, nv, m, [&](int64_t i, int64_t v) {
+        const int64_t s = slot[v], t = s / TILE_V;
         const uint32_t row = (uint32_t)(s % TILE_V), a = atom[i];
         key[i] = order == BY_TABLE ? ((uint64_t)tile_brick[t] << bf) | (uint64_t)fasc[i]
                  : order == BY_DSC ? ((uint64_t)t << 16) | ((a >> 7) << 14) | dsc_cell(a, row)
                                    : ((uint64_t)t << 16) | ((row >> 5) << 14) | (a << 5) | (row & 31u);
         payload[i] = (uint32_t)i;
-    }
+    });
 }
 
 // Offsets of the bricks' tables from the sorted (brick, fascicle) keys.
@@ -890,7 +884,7 @@ static life_status sort_entries(const life_index_s* ix, const TileSet& H, const 
     const int64_t m = ix->nnz;
     LIFE_TRY(key.alloc(sizeof(uint64_t) * m, s));
     LIFE_TRY(pay.alloc(sizeof(uint32_t) * m, s));
-    entry_key_kernel<<<grid1d(m), 256, 0, s>>>(ix->vox.vox_ptr.as<int32_t>(), ix->nv, slot.as<int64_t>(),
+    entry_key_kernel<<<entry_segments_grid(m), 256, 0, s>>>(ix->vox.vox_ptr.as<int32_t>(), ix->nv, slot.as<int64_t>(),
                                                H.tile_brick.as<int32_t>(), ix->vox.atom.as<uint16_t>(),
                                                ix->vox.fasc.as<int32_t>(), m, order, ix->key_bits_f, key.as<uint64_t>(),
                                                pay.as<uint32_t>());
