@@ -36,10 +36,11 @@ PEAK_FALLBACK = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0}
 # fused residual = preparation launch + DSC kernel; WC through the public call =
 # max|r| and preparation launch + WC kernel; per path (BF16 storage, FP32 storage on the
 # tensor cores).  Scaled to the timed workload by its entry count (the traffic
-# grows with the entries and voxels alike).  The figures hold only for the kernel
-# source that was captured; after any change to it the bench reports null.
+# grows with the entries and voxels alike).  The figures hold only for the sources that
+# were captured (the kernels, the layout they read and the rules that shape a launch,
+# hashed together); after any change to one of them the bench reports null.
 TRAFFIC_CAPTURE = {
-    "src": os.path.join("paper_1905_06234_gb300", "csrc", "spmv_tc.cu"),
+    "src": ["spmv_tc.cu", "tile_build.cu", "tile_layout.cuh", "launch_rules.cuh", "tc_ptx.cuh", "life_internal.cuh"],
     "sha256": "08e64cd0fa52498f90317c2407f4bd2e98f22266e4a9500bef050c5b7a6ed5e8",
     "nnz": 23816750,
     "bytes": {
@@ -49,18 +50,25 @@ TRAFFIC_CAPTURE = {
 }
 
 
+def traffic_digest():
+    """One SHA-256 of the sources the traffic figures depend on, in their listed order."""
+    import hashlib
+    h = hashlib.sha256()
+    for name in TRAFFIC_CAPTURE["src"]:
+        with open(os.path.join(ROOT, "paper_1905_06234_gb300", "csrc", name), "rb") as fh:
+            h.update(hashlib.sha256(fh.read()).digest())
+    return h.hexdigest()
+
+
 def kernel_traffic(path_name, kind, nnz):
     """Measured DRAM bytes of one launch (scaled to `nnz` entries if the workload differs), or None."""
-    import hashlib
     per_path = TRAFFIC_CAPTURE["bytes"].get(path_name)
     if per_path is None:
         return None
     try:
-        with open(os.path.join(ROOT, TRAFFIC_CAPTURE["src"]), "rb") as fh:
-            sha = hashlib.sha256(fh.read()).hexdigest()
+        if traffic_digest() != TRAFFIC_CAPTURE["sha256"]:
+            return None
     except OSError:
-        return None
-    if sha != TRAFFIC_CAPTURE["sha256"]:
         return None
     return per_path[kind] * nnz / TRAFFIC_CAPTURE["nnz"]
 
