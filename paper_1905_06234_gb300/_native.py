@@ -150,10 +150,17 @@ def _ptr(t):
     return t.data_ptr()   # a plain address: the argument types make a pointer of it
 
 
+# The raw handle of the current stream: a small call (11 us on the GPU) is bound by the
+# host, and the stream object torch.cuda.current_stream() makes is most of what this
+# module adds to it.  The binding is not part of torch's public interface; without it
+# the stream object serves.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream():
-    # the raw handle: a small call (11 us on the GPU) is bound by the host, and the stream
-    # object torch.cuda.current_stream() makes is most of what this module adds to it
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _need(t, dtype, numel, name):
