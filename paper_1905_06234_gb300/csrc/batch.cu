@@ -368,9 +368,6 @@ extern "C" life_status life_batch_create(int32_t n, const life_index* idx, const
         bi.vox_off[p] = (int32_t)voff[p];
         bi.fasc_off[p] = (int32_t)foff[p];
     }
-    bi.vox_group.resize(voff[n]);
-    for (int p = 0; p < n; ++p)
-        for (int64_t v = voff[p]; v < voff[p + 1]; ++v) bi.vox_group[v] = p;
     const int algo = o.algo != LIFE_ALGO_AUTO ? o.algo : idx[0]->algo;
     life_status st = build_index_layouts(ix, atom.as<int32_t>(), voxel.as<int32_t>(), fasc.as<int32_t>(),
                                          val.as<float>(), all_ijk ? ijk.as<int32_t>() : nullptr, algo, s);

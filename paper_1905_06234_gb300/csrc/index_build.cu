@@ -111,14 +111,14 @@ life_status exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t n, cudaS
 // writes, so that a warp writes a few runs of consecutive pairs instead of 32
 // scattered ones (32-byte sectors of which 12 B were used): 6144 pairs a tile give
 // runs of 24 pairs at 8 bits, 48 at 7, and two CTAs of 512 threads share an SM.
-// The index build of the paper-scale workload (80M entries, BF16 storage) took
-// 80.0 ms with 22 passes of an unstaged scatter (1.9 ms each), 44.0 ms with this
-// one, 16 passes (the callers sort only the bits that are not in order yet) and
-// the merge below in two passes.
+// A new index of the paper-scale workload (80M entries, BF16 storage) with its first
+// DSC and WC took 80.0 ms with 22 passes of an unstaged scatter (1.9 ms each), 44.0 ms
+// with this one, 16 passes (the callers sort only the bits that are not in order yet)
+// and the merge below in two passes; 16.4 ms since the tile layout is counted.
 
 constexpr int RS_THREADS = 512;
 constexpr int RS_WARPS = RS_THREADS / 32;
-constexpr int RS_ROUNDS = 12;                     // items per lane (16 spill; paper-scale build 14.7 ms, with 12 14.3)
+constexpr int RS_ROUNDS = 12;                     // items per lane (16 spill: the paper-scale build alone 14.7 ms, 14.1 with 12)
 constexpr int RS_TILE = RS_THREADS * RS_ROUNDS;   // 6144 items per block
 constexpr int RS_DIGITS = 256;
 constexpr int RS_COPIES = 8;                      // histogram copies: two warps add to each
@@ -152,7 +152,7 @@ rs_scatter_kernel(const uint64_t* __restrict__ kin, const uint32_t* __restrict__
     extern __shared__ __align__(16) unsigned char rs_smem[];
     uint64_t* sk = reinterpret_cast<uint64_t*>(rs_smem);
     uint32_t* sv = reinterpret_cast<uint32_t*>(sk + RS_TILE);
-    uint16_t* wcnt = reinterpret_cast<uint16_t*>(sv + RS_TILE);  // [warp][digit]: at most 512 items a warp
+    uint16_t* wcnt = reinterpret_cast<uint16_t*>(sv + RS_TILE);  // [warp][digit]: at most 384 items a warp
     __shared__ int32_t gofs[RS_DIGITS], wtot[RS_DIGITS / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int i = tid; i < RS_WARPS * RS_DIGITS / 2; i += RS_THREADS) reinterpret_cast<uint32_t*>(wcnt)[i] = 0u;

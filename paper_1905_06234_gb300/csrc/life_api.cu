@@ -74,7 +74,7 @@ life_status spmv_wc(life_index_s* ix, const float* D, const float* r, float* g, 
 }
 
 // Builds every layout of an index whose sizes, precision, brick_dim (and, for a
-// batch, batch.vox_off / batch.vox_group) the caller has set.  algo_req is the
+// batch, batch.n and batch.vox_off) the caller has set.  algo_req is the
 // requested LIFE_ALGO_*; AUTO picks the tensor-core path for BF16 storage and
 // falls back to the CUDA-core kernels when the tile layout is not supported.
 life_status build_index_layouts(life_index_s* ix, const int32_t* atom, const int32_t* voxel, const int32_t* fasc,

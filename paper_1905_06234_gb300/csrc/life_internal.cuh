@@ -212,7 +212,6 @@ struct BatchInfo {
     int32_t n = 0;
     std::vector<int32_t> vox_off, fasc_off;  // host [n+1]
     std::vector<int64_t> nnz_off;            // host [n+1] merged entries
-    std::vector<int32_t> vox_group;          // host [Nv] problem of each voxel (tile grouping)
     DevBuf d_vox_off, d_fasc_off;            // int32 [n+1]
     DevBuf brick_prob;                       // TC: int32 [n_bricks] problem of each brick
     int32_t tc_grid = 0;                     // TC: CTAs of a batched SpMV launch

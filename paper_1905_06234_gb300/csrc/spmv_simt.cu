@@ -823,9 +823,11 @@ life_status grad_D_simt(life_index_s* ix, const float* gy, const float* w, float
 //
 // life_dsc_grad_D_noalloc: the same two kernels as life_dsc_grad_D, with the
 // split-K partial sums in a fixed device array compiled into this library
-// instead of memory allocated per call.  It serves callers that may not
-// allocate device memory while they run (for example code being captured into a
-// CUDA graph, or an allocation-free real-time loop).
+// instead of memory of the index (nnz / 256 · Nθ floats, about 120 MB at the
+// paper's scale, which life_dsc_grad_D's first call allocates and the index keeps).
+// It serves callers that may not allocate device memory while they run (for
+// example code being captured into a CUDA graph, or an allocation-free real-time
+// loop).
 
 #include <mutex>
 

@@ -62,7 +62,7 @@ __device__ __forceinline__ void block_absmax_out(uint32_t m, uint32_t* out) {
 // The sparse-w-aware DSC (Sec. 4.2.1: an entry whose weight is zero contributes
 // nothing, and SBB-NNLS iterates keep many weights at exactly zero).  Besides the
 // full stream, the index keeps a compacted copy holding only the entries of a
-// live set L of brick-local fascicles, with the same (tile, 32-atom sub-chunk)
+// live set L of brick-local fascicles, with the same (tile, 128-atom chunk)
 // structure.  Every DSC call checks on the device whether the input's support
 // lies inside L ("stale" otherwise); a small decision kernel then picks the full
 // or the compacted stream for this call, and may rebuild the compacted stream
@@ -359,7 +359,7 @@ struct TcArgs {
     const float* D;
     const float* x;      // DSC: w [Nf];   WC: r [Nθ·Nv]
     const float* b;      // DSC residual or NULL
-    float* out;          // DSC: y (or NULL);   WC: g (zeroed by the caller)
+    float* out;          // DSC: y (or NULL);   WC: g (zeroed by the launch before)
     double* partial;     // DSC: per-CTA FP64 Σ out²
     const float* val32;  // DSC on an FP32-storage index: the stream's values (val is then unused)
     const float* wval32; // WC on an FP32-storage index: the WC stream's values (wval is then unused)
@@ -939,9 +939,8 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
             int vw = warp;  // the warp's place in the chunk: it takes block vw first
             uint32_t st = 0, ph = 0;
             int base = (beg & ~7) + tid * SLOT;
-            bool have = base < end;
             SlotT cur{};
-            if (have) load_slot(A.soff, A, base, cur);
+            if (base < end) load_slot(A.soff, A, base, cur);
             bool new_brick = true, dead = false;
             uint32_t tab_ph = 0, tab_n = 0;
             for (;;) {
@@ -1055,7 +1054,6 @@ __global__ void __maxnreg__(72) dsc_tc_kernel(TcArgs A) {
                 end = nend;
                 new_brick = nnew;
                 base = nbase;
-                have = nhave;
                 cur = nxt;  // an empty slot when this lane has none in the next chunk
             }
             // no bulk table copy may still be writing shared memory when the CTA exits

@@ -10,13 +10,13 @@
 // them.  Every entry is read a few times (2 to 6 B each) and written once per
 // stream.  Sorting (key, position) pairs instead, as radix passes of 24 B a pair
 // with the streams gathered through the positions afterwards, moved about ten
-// times as much: for the paper-scale workload (80M entries, BF16 storage) the
-// whole index build took 44.0 ms that way and takes 16.6 ms now, of which the
-// bricks' tables are 1.3 ms and the streams 3.1 ms (bound by the latency of a
-// pass: one 1024-thread CTA an SM, since a pass's cells and entries fill its
-// shared memory).  (Sorting stays the better way for some shapes: see sort_is_faster.)
-// The host's part of the old build (a stable sort of the voxels,
-// copies both ways) went with it.
+// times as much: for the paper-scale workload (80M entries, BF16 storage) a new index
+// with its first DSC and WC took 44.0 ms that way and takes 16.4 ms now (14.1 ms the
+// build alone), of which the bricks' tables are 1.3 ms and the streams 3.1 ms (bound by
+// the latency of a pass: one 1024-thread CTA an SM, since a pass's cells and entries
+// fill its shared memory).  The host's part of the old build (a stable sort of the
+// voxels, copies both ways) went with it.  Some shapes are still sooner sorted: see
+// sort_is_faster.
 #include <algorithm>
 #include <cstring>
 #include <numeric>
@@ -62,7 +62,6 @@ __device__ __forceinline__ uint32_t dsc_cell(uint32_t a, uint32_t row) {
 
 struct BrickShape {
     int x, y, z;
-    int64_t volume() const { return (int64_t)x * y * z; }
 };
 
 // Largest coordinate along each axis (at least 0).
@@ -799,7 +798,7 @@ struct TileSet {
 static life_status assign_tiles(const life_index_s* ix, const std::vector<BrickShape>& shape, TileSet& H,
                                 cudaStream_t s) {
     const int64_t nv = ix->nv;
-    const bool grouped = !ix->batch.vox_group.empty();
+    const bool grouped = ix->batch.n > 0;
     const int ng = (int)shape.size();
     std::vector<int32_t> hshape;
     for (const BrickShape& b : shape) hshape.insert(hshape.end(), {b.x, b.y, b.z});
@@ -1084,13 +1083,14 @@ life_status build_tile_layout(life_index_s* ix, cudaStream_t s) {
     // table overflows halves its brick's largest dimension and the bricks are
     // formed again, until all groups fit (other groups keep their bricks).
     const int B0 = std::max(2, ix->brick_dim);
-    const bool grouped = !ix->batch.vox_group.empty();
+    const bool grouped = ix->batch.n > 0;
     const int ngroups = grouped ? ix->batch.n : 1;
     std::vector<BrickShape> shape(ngroups, BrickShape{B0, B0, B0});
     for (int attempt = 0; attempt < 32 && !ok; ++attempt) {
         LIFE_TRY(assign_tiles(ix, shape, H, s));
         const int bt = nbits64(H.n_tiles), bb = nbits64(H.n_bricks);
-        if (bt + 16 + bf > 64 || bb + bf > 64) {
+        if (bt + 16 + bf > 64 || bb + bf > 64) {  // (brick, fascicle) is a sort key of the sorted form;
+                                                  // the other has been a limit of the layout all along
             set_error("tensor-core layout: sort key too wide");
             return LIFE_ENOTSUP;
         }
