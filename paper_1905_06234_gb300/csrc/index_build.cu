@@ -502,10 +502,18 @@ life_status build_voxel_layout(life_index_s* ix, const int32_t* atom, const int3
 
 // ------------------------------------------------------------ re-sorting
 
-// Voxel of each entry of the merged list.
-__global__ void entry_voxel_kernel(const int32_t* __restrict__ vox_ptr, int32_t nv, int64_t m,
-                                   int32_t* __restrict__ voxel) {
-    for_entry_segments(vox_ptr, nv, m, [&](int64_t i, int64_t v) { voxel[i] = (int32_t)v; });
+// The merged list in its own order, the voxel of each entry from the voxels' offsets
+// (outputs that are NULL are left out).
+__global__ void list_export_kernel(const int32_t* __restrict__ vox_ptr, int32_t nv, const uint16_t* __restrict__ asrc,
+                                   const int32_t* __restrict__ fsrc, const float* __restrict__ xsrc, int64_t m,
+                                   int32_t* __restrict__ atom, int32_t* __restrict__ voxel,
+                                   int32_t* __restrict__ fasc, float* __restrict__ val) {
+    for_entry_segments(vox_ptr, nv, m, [&](int64_t i, int64_t v) {
+        if (atom) atom[i] = asrc[i];
+        if (voxel) voxel[i] = (int32_t)v;
+        if (fasc) fasc[i] = fsrc[i];
+        if (val) val[i] = xsrc[i];
+    });
 }
 
 // Re-keys the merged (v, a, f) list in another order; payload = merged position.
@@ -525,7 +533,7 @@ __global__ void gather_export_kernel(const int32_t* __restrict__ vsrc, const uin
                                      int32_t* __restrict__ voxel, int32_t* __restrict__ fasc,
                                      float* __restrict__ val) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t p = perm ? perm[i] : (uint32_t)i;
+        const uint32_t p = perm[i];
         if (atom) atom[i] = asrc[p];
         if (voxel) voxel[i] = vsrc[p];
         if (fasc) fasc[i] = fsrc[p];
@@ -533,10 +541,9 @@ __global__ void gather_export_kernel(const int32_t* __restrict__ vsrc, const uin
     }
 }
 
-// Sorted permutation of the merged list for a layout (NULL perm = voxel order).
+// Sorted permutation of the merged list for a layout other than its own.
 static life_status layout_perm(life_index_s* ix, int layout, const int32_t* voxel, TmpBuf& perm, cudaStream_t s) {
     const int64_t m = ix->nnz;
-    if (layout == LIFE_LAYOUT_VOXEL || m == 0) return LIFE_OK;
     TmpBuf keys;
     LIFE_TRY(keys.alloc(sizeof(uint64_t) * m, s));
     LIFE_TRY(perm.alloc(sizeof(uint32_t) * m, s));
@@ -559,21 +566,25 @@ life_status export_layout(life_index_s* ix, int layout, int32_t* atom, int32_t* 
     }
     const int64_t m = ix->nnz;
     if (m == 0) return LIFE_OK;
-    // the voxel of each entry: straight into the output in the list's own order, else
-    // through a temporary that the permutation reads
-    const bool own = layout == LIFE_LAYOUT_VOXEL;
-    TmpBuf vox, perm;
-    if (!own) LIFE_TRY(vox.alloc(sizeof(int32_t) * m, s));
-    int32_t* vdst = own ? voxel : vox.as<int32_t>();
-    if (vdst) {
-        entry_voxel_kernel<<<entry_segments_grid(m), 256, 0, s>>>(ix->vox.vox_ptr.as<int32_t>(), ix->nv, m, vdst);
-        LIFE_CHECK_LAUNCH();
-    }
-    LIFE_TRY(layout_perm(ix, layout, vox.as<int32_t>(), perm, s));
     const float* x = ix->precision == LIFE_BF16 ? ix->uval.as<float>() : ix->vox.val.as<float>();
+    if (layout == LIFE_LAYOUT_VOXEL) {  // the list's own order
+        list_export_kernel<<<entry_segments_grid(m), 256, 0, s>>>(ix->vox.vox_ptr.as<int32_t>(), ix->nv,
+                                                                  ix->vox.atom.as<uint16_t>(),
+                                                                  ix->vox.fasc.as<int32_t>(), x, m, atom, voxel, fasc,
+                                                                  val);
+        LIFE_CHECK_LAUNCH();
+        LIFE_CUDA_TRY(cudaStreamSynchronize(s));
+        return LIFE_OK;
+    }
+    TmpBuf vox, perm;
+    LIFE_TRY(vox.alloc(sizeof(int32_t) * m, s));
+    list_export_kernel<<<entry_segments_grid(m), 256, 0, s>>>(ix->vox.vox_ptr.as<int32_t>(), ix->nv, nullptr, nullptr,
+                                                              nullptr, m, nullptr, vox.as<int32_t>(), nullptr, nullptr);
+    LIFE_CHECK_LAUNCH();
+    LIFE_TRY(layout_perm(ix, layout, vox.as<int32_t>(), perm, s));
     gather_export_kernel<<<grid_for(m), 256, 0, s>>>(vox.as<int32_t>(), ix->vox.atom.as<uint16_t>(),
                                                      ix->vox.fasc.as<int32_t>(), x, perm.as<uint32_t>(), m, atom,
-                                                     own ? nullptr : voxel, fasc, val);
+                                                     voxel, fasc, val);
     LIFE_CHECK_LAUNCH();
     LIFE_CUDA_TRY(cudaStreamSynchronize(s));
     return LIFE_OK;

@@ -284,23 +284,19 @@ __global__ void widen_bf16_kernel(const __nv_bfloat16* __restrict__ in, int64_t 
         out[i] = __bfloat162float(in[i]);
 }
 
-// The exported form of the DSC stream's fascicle field: the brick-local fascicle
-// (the stream holds its byte offset in the weight table) | 0x8000 when the entry
-// continues the previous entry's (atom, row) (the stream keeps that bit in soff).
-__global__ void export_fl_kernel(const uint16_t* __restrict__ fl, const uint16_t* __restrict__ soff, int64_t n,
-                                 uint16_t* __restrict__ out) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = (uint16_t)((fl[i] >> 2) | (soff[i] & CONT));
-}
-
-// row | atom << 7 of each DSC-stream entry: the cell from its S byte offset, the
-// 128-atom chunk from the entry's place in chunk_ptr (n_seg chunks, n_c per tile).
-__global__ void export_va_kernel(const uint16_t* __restrict__ soff, const int32_t* __restrict__ chunk_ptr,
-                                 int64_t n_seg, int n_c, int64_t n, uint16_t* __restrict__ out) {
+// The exported forms of the DSC stream's fields (either may be left out).  va: row |
+// atom << 7, the cell from its S byte offset, the 128-atom chunk from the entry's place in
+// chunk_ptr (n_seg chunks, n_c per tile).  fl: the brick-local fascicle (the stream holds
+// its byte offset in the weight table) | 0x8000 when the entry continues the previous
+// entry's (atom, row) (the stream keeps that bit in soff).
+__global__ void export_cells_kernel(const uint16_t* __restrict__ soff, const uint16_t* __restrict__ fl,
+                                    const int32_t* __restrict__ chunk_ptr, int64_t n_seg, int n_c, int64_t n,
+                                    uint16_t* __restrict__ va_out, uint16_t* __restrict__ fl_out) {
     for_entry_segments(chunk_ptr, n_seg, n, [&](int64_t i, int64_t s) {
-        const uint32_t so = soff[i] & 0x7FFFu;
+        const uint32_t k = soff[i], so = k & 0x7FFFu;
         const uint32_t row = (so >> 11) * 8 + ((so >> 4) & 7u), a = ((so >> 7) & 15u) * 8 + ((so >> 1) & 7u);
-        out[i] = (uint16_t)(row | ((a + (uint32_t)s % (uint32_t)n_c * DKC) << 7));
+        if (va_out) va_out[i] = (uint16_t)(row | ((a + (uint32_t)s % (uint32_t)n_c * DKC) << 7));
+        if (fl_out) fl_out[i] = (uint16_t)((fl[i] >> 2) | (k & CONT));
     });
 }
 
@@ -318,13 +314,10 @@ life_status export_tiles(life_index_s* ix, int32_t* tile_vox, int32_t* chunk_ptr
     LIFE_TRY(cp(brick_fasc_ptr, L.brick_fasc_ptr, sizeof(int32_t) * (L.n_bricks + 1)));
     LIFE_TRY(cp(brick_fasc, L.brick_fasc, L.brick_fasc.bytes));
     LIFE_TRY(cp(brick_order, L.brick_order, sizeof(int32_t) * L.n_bricks));
-    if (va && L.n_nnz > 0) {
-        export_va_kernel<<<entry_segments_grid(L.n_nnz), 256, 0, s>>>(L.soff.as<uint16_t>(), L.chunk_ptr.as<int32_t>(),
-                                                              L.n_tiles * (L.kp / DKC), L.kp / DKC, L.n_nnz, va);
-        LIFE_CHECK_LAUNCH();
-    }
-    if (fl && L.n_nnz > 0) {
-        export_fl_kernel<<<grid1d(L.n_nnz), 256, 0, s>>>(L.fl.as<uint16_t>(), L.soff.as<uint16_t>(), L.n_nnz, fl);
+    if ((va || fl) && L.n_nnz > 0) {
+        export_cells_kernel<<<entry_segments_grid(L.n_nnz), 256, 0, s>>>(
+            L.soff.as<uint16_t>(), L.fl.as<uint16_t>(), L.chunk_ptr.as<int32_t>(), L.n_tiles * (L.kp / DKC), L.kp / DKC,
+            L.n_nnz, va, fl);
         LIFE_CHECK_LAUNCH();
     }
     if (val && L.n_nnz > 0) {
