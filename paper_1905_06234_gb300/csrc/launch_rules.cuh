@@ -108,13 +108,12 @@ inline WorkShare share_out(const std::vector<int32_t>& order, const std::vector<
 // it fits beside the brick table and two S stages, and rows are 16-byte aligned: can);
 // stages: S stages.  The lines, from DSC calls timed in each form (us, one GB300; entries
 // per tile and 128-atom chunk):
-//  - The tile of Y saves the epilogue's reads of b, which a tile of several chunks hides
-//    behind nothing (64^3 voxels, Nθ 96, Na 360: 339 entries 128 -> 106, 3812 177 -> 146,
-//    and 40^3 at 7621 the same either way).  A tile of one chunk is over before its b has
-//    arrived (Nθ 64, Na 128: 1005 81 -> 87, 7536 106 -> 109, 16351 132 -> 123, 22635 160 ->
-//    140): it takes the tile from 16384 entries on.  Bricks of one tile gather a table for
-//    every tile, and there the copies only delay (4^3 bricks, 48^3 voxels: 1270 112 -> 104,
-//    2752 126 -> 129, 4978 147 -> 167): up to 2304.
+//  - The tile of Y spares the epilogue its reads of b, a few at a time (64^3 voxels, Nθ 96,
+//    Na 360: 339 entries 128 -> 106, 3812 177 -> 146).  A tile of one chunk is over before
+//    its b has arrived (Nθ 64, Na 128: 1005 81 -> 87, 7536 106 -> 109, 16351 132 -> 123,
+//    22635 160 -> 140): it takes the tile of Y from 16384 entries on.  Bricks of one tile
+//    gather a table for every tile, and the copies come on top of that (4^3 bricks, 48^3
+//    voxels: 1270 112 -> 104, 2752 126 -> 129, 4978 147 -> 167): up to 2304 entries.
 //  - A third and fourth stage let idle producers start on the next chunks: worth it where
 //    a chunk's 256-entry blocks are for at most half of the 23 producer warps and a tile has
 //    more than two chunks (64^3, Nθ 32, Na 512: 255 105 -> 81, 2864 137 -> 135, 7481 208 ->

@@ -803,7 +803,7 @@ __global__ void __launch_bounds__(PREP_THREADS) tc_prep_kernel(PrepArgs P) {
 //  - the tile's rows of b are bulk-copied into shared memory while its S is formed, b
 //    is subtracted from Y in place there and Y bulk-copied out: the epilogue's reads of
 //    b, a few 16-byte loads a thread at a time, took 7 us of the 8 us a tile had;
-//  - up to four S stages as they fit, and the warp that takes a chunk's first block
+//  - up to four S stages, and the warp that takes a chunk's first block
 //    moves on by DSC_ROT from chunk to chunk (the same three of the 23 producers had
 //    all the work).
 // 64^3 workload: 130 -> 108 us with b, an iteration 418 -> 367 us.  Where it is taken, and
