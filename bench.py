@@ -41,11 +41,11 @@ PEAK_FALLBACK = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0}
 # hashed together); after any change to one of them the bench reports null.
 TRAFFIC_CAPTURE = {
     "src": ["spmv_tc.cu", "tile_build.cu", "tile_layout.cuh", "launch_rules.cuh", "tc_ptx.cuh", "life_internal.cuh"],
-    "sha256": "08e64cd0fa52498f90317c2407f4bd2e98f22266e4a9500bef050c5b7a6ed5e8",
+    "sha256": "41cb72855ae39d33c93443b60d70790e1bec59391817385c4b132b8cd07d518c",
     "nnz": 23816750,
     "bytes": {
-        "bf16-tc": {"dsc": (762112 + 0) + (197602560 + 16938240), "wc": (40148224 + 7936) + (201893376 + 47104)},
-        "fp32-tc": {"dsc": (761856 + 0) + (248656896 + 19802880), "wc": (40147968 + 0) + (256412416 + 117248)},
+        "bf16-tc": {"dsc": (761856 + 0) + (197695488 + 16835328), "wc": (40148224 + 256) + (201898240 + 80384)},
+        "fp32-tc": {"dsc": (761600 + 0) + (248741632 + 19769088), "wc": (40147968 + 0) + (256169216 + 425472)},
     },
 }
 
