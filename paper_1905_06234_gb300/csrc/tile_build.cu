@@ -791,6 +791,7 @@ static life_status download(std::vector<T>& dst, const void* src, size_t n, cuda
 // Bricks and tiles of one attempt (device arrays, sizes on the host).
 struct TileSet {
     DevBuf tile_vox, tile_brick, brick_tile_ptr, brick_group;
+    std::vector<int32_t> btile;  // host copy of brick_tile_ptr
     int64_t n_tiles = 0;
     int32_t n_bricks = 0;
 };
@@ -857,10 +858,9 @@ static life_status assign_tiles(const life_index_s* ix, const std::vector<BrickS
     brick_ntiles_kernel<<<grid1d((int64_t)nb + 1), 256, 0, s>>>(start.as<int32_t>(), nb, nt.as<int32_t>());
     LIFE_CHECK_LAUNCH();
     LIFE_TRY(exclusive_scan_i32(nt.as<int32_t>(), H.brick_tile_ptr.as<int32_t>(), (int64_t)nb + 1, s));
-    int32_t n_tiles = 0;
-    LIFE_CUDA_TRY(cudaMemcpyAsync(&n_tiles, H.brick_tile_ptr.as<int32_t>() + nb, 4, cudaMemcpyDeviceToHost, s));
+    LIFE_TRY(download(H.btile, H.brick_tile_ptr.p, (size_t)nb + 1, s));
     LIFE_CUDA_TRY(cudaStreamSynchronize(s));
-    H.n_tiles = n_tiles;
+    H.n_tiles = H.btile[nb];
     LIFE_TRY(H.tile_vox.alloc(sizeof(int32_t) * H.n_tiles * TILE_V));
     LIFE_TRY(H.tile_brick.alloc(sizeof(int32_t) * H.n_tiles));
     LIFE_CUDA_TRY(cudaMemsetAsync(H.tile_vox.p, 0xFF, sizeof(int32_t) * H.n_tiles * TILE_V, s));
@@ -972,8 +972,8 @@ static life_status sort_tables_and_streams(life_index_s* ix, const TileSet& H, S
 // counted / sorted: 80M entries in 500k voxels 15.7 / 30.0 ms, 10M in 32768 voxels 3.5 /
 // 5.3; 3M in 4096 2.9 / 2.9, 6M there 4.6 / 3.8; 1M in 128 25 / 1.8, 10M in 128 1515 /
 // 4.8; 50M in 4M voxels with 5M fascicles 29.7 / 22.0, with 50M fascicles 120 / 23.
-static bool sort_is_faster(const std::vector<int32_t>& base, const std::vector<int32_t>& quarter,
-                           const std::vector<int32_t>& btile, int n_c, bool wc, int64_t nf, int window, int num_sms) {
+static bool sort_is_faster(const int32_t* base, const int32_t* quarter, const std::vector<int32_t>& btile, int n_c,
+                           bool wc, int64_t nf, int window, int num_sms) {
     constexpr double PASS = 9.0, WALK = 5.0e-4, WINDOW = 9.0, TABLE_WALK = 8.0e-4, ROWS_WALK = 0.012, SORT = 500.0,
                      SORT_ENTRY = 2.5e-4;
     const double sms = std::max(num_sms, 1), windows = (double)((nf + window - 1) / window);
@@ -993,7 +993,7 @@ static bool sort_is_faster(const std::vector<int32_t>& base, const std::vector<i
         tab += us;
         tab_max = std::max(tab_max, us);
     }
-    return std::max(tab_max, tab / sms) + std::max(str_max, str / sms) > SORT + SORT_ENTRY * base.back();
+    return std::max(tab_max, tab / sms) + std::max(str_max, str / sms) > SORT + SORT_ENTRY * base[btile.back()];
 }
 
 template <class VT>
@@ -1073,8 +1073,8 @@ life_status build_tile_layout(life_index_s* ix, cudaStream_t s) {
     const int bf = ix->key_bits_f;
     TileSet H;
     SortedTables ST;
-    std::vector<int32_t> hbptr, hgroup, hbase, hquarter, hbtile;
-    TmpBuf count, tcount, tquarter, tbase;
+    std::vector<int32_t> hbptr, hgroup, htile;  // htile: [n_tiles + 1] entry offsets, then the fullest quarters
+    TmpBuf count, tcount, tinfo;                // tinfo: htile on the device
     bool ok = false, sorted = false;
     const int window = bt_window(ix->nf);
     const size_t csm = (size_t)window / 8;
@@ -1095,18 +1095,16 @@ life_status build_tile_layout(life_index_s* ix, cudaStream_t s) {
             return LIFE_ENOTSUP;
         }
         LIFE_TRY(tcount.alloc(sizeof(int32_t) * (H.n_tiles + 1), s));
-        LIFE_TRY(tquarter.alloc(sizeof(int32_t) * (H.n_tiles + 1), s));
-        LIFE_TRY(tbase.alloc(sizeof(int32_t) * (H.n_tiles + 1), s));
+        LIFE_TRY(tinfo.alloc(2 * sizeof(int32_t) * (H.n_tiles + 1), s));
         tile_count_kernel<<<(unsigned)((H.n_tiles + 8) / 8), 256, 0, s>>>(
             H.tile_vox.as<int32_t>(), ix->vox.vox_ptr.as<int32_t>(), H.n_tiles, tcount.as<int32_t>(),
-            tquarter.as<int32_t>());
+            tinfo.as<int32_t>() + H.n_tiles + 1);
         LIFE_CHECK_LAUNCH();
-        LIFE_TRY(exclusive_scan_i32(tcount.as<int32_t>(), tbase.as<int32_t>(), H.n_tiles + 1, s));
-        LIFE_TRY(download(hbase, tbase.p, (size_t)H.n_tiles + 1, s));
-        LIFE_TRY(download(hquarter, tquarter.p, (size_t)H.n_tiles, s));
-        LIFE_TRY(download(hbtile, H.brick_tile_ptr.p, (size_t)H.n_bricks + 1, s));
+        LIFE_TRY(exclusive_scan_i32(tcount.as<int32_t>(), tinfo.as<int32_t>(), H.n_tiles + 1, s));
+        LIFE_TRY(download(htile, tinfo.p, 2 * ((size_t)H.n_tiles + 1), s));
         LIFE_CUDA_TRY(cudaStreamSynchronize(s));
-        sorted = m > 0 && sort_is_faster(hbase, hquarter, hbtile, L.kp / DKC, L.wc_stream, ix->nf, window, ix->num_sms);
+        sorted = m > 0 && sort_is_faster(htile.data(), htile.data() + H.n_tiles + 1, H.btile, L.kp / DKC, L.wc_stream,
+                                         ix->nf, window, ix->num_sms);
         L.brick_fasc_ptr.release();
         LIFE_TRY(L.brick_fasc_ptr.alloc(sizeof(int32_t) * ((size_t)H.n_bricks + 1)));
         if (sorted) {
@@ -1192,9 +1190,9 @@ life_status build_tile_layout(life_index_s* ix, cudaStream_t s) {
     LIFE_CUDA_TRY(cudaMemsetAsync(rv.p, 0, sizeof(uint32_t), s));
     SortedTables* st = sorted ? &ST : nullptr;
     if (L.vbytes == 4)
-        LIFE_TRY(build_tables_and_streams<float>(ix, H, tbase.as<int32_t>(), window, st, rv.as<uint32_t>(), s));
+        LIFE_TRY(build_tables_and_streams<float>(ix, H, tinfo.as<int32_t>(), window, st, rv.as<uint32_t>(), s));
     else
-        LIFE_TRY(build_tables_and_streams<__nv_bfloat16>(ix, H, tbase.as<int32_t>(), window, st, rv.as<uint32_t>(), s));
+        LIFE_TRY(build_tables_and_streams<__nv_bfloat16>(ix, H, tinfo.as<int32_t>(), window, st, rv.as<uint32_t>(), s));
     std::vector<int32_t> wptr(H.n_bricks + 1, 0);
     {
         // padded, 16-byte aligned per-brick weight slots for the DSC's bulk table loads
@@ -1250,12 +1248,12 @@ life_status build_tile_layout(life_index_s* ix, cudaStream_t s) {
     std::memcpy(&L.run_vmax, &vbits, sizeof(float));
     std::vector<int64_t> bnnz(H.n_bricks);
     for (int64_t b = 0; b < H.n_bricks; ++b)
-        bnnz[b] = (int64_t)hbase[hbtile[b + 1]] - hbase[hbtile[b]] + 64 * (hbtile[b + 1] - hbtile[b]);
+        bnnz[b] = (int64_t)htile[H.btile[b + 1]] - htile[H.btile[b]] + 64 * (H.btile[b + 1] - H.btile[b]);
     std::vector<int32_t> order(H.n_bricks);
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return bnnz[x] > bnnz[y]; });
     LIFE_TRY(upload(L.brick_order, order, s));
-    const WorkShare W = share_out(order, hbtile, hbase, hbptr, ix->num_sms, grouped, L.vbytes == 4);
+    const WorkShare W = share_out(order, H.btile, htile, hbptr, ix->num_sms, grouped, L.vbytes == 4);
     L.grid = W.grid();
     L.n_units = (int32_t)W.brick.size();
     std::vector<int32_t> units = W.cta_unit;

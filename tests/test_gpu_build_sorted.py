@@ -133,17 +133,17 @@ def test_many_fascicles_bit_exact(life):
 
 
 def build_s(life, n, nv, nf, seed=1):
-    """Median build time of n random entries (sorted by fascicle), BF16 on the tensor cores."""
+    """Shortest build time of n random entries (sorted by fascicle), BF16 on the tensor cores."""
     g = torch.Generator(device="cuda").manual_seed(seed)
     ints = lambda k: torch.randint(0, k, (n,), generator=g, device="cuda", dtype=torch.int32)
     a, v, f = ints(360), ints(nv), ints(nf).sort()[0]
     x, t = torch.rand(n, generator=g, device="cuda") + 0.5, []
-    for _ in range(4):
+    for _ in range(6):
         torch.cuda.synchronize()
         t0 = time.perf_counter()
         life.life_build_index(a, v, f, x, 16, 360, nv, nf, precision=life.LIFE_BF16, algo=life.LIFE_ALGO_TC).close()
         t.append(time.perf_counter() - t0)
-    return sorted(t[1:])[1]
+    return min(t[1:])
 
 
 def test_full_tiles_build_as_fast(life):

@@ -16,7 +16,7 @@ def life():
     return L
 
 
-def median_s(f):
+def best_s(f):
     t = []
     for _ in range(12):
         torch.cuda.synchronize()
@@ -24,7 +24,7 @@ def median_s(f):
         f()
         torch.cuda.synchronize()
         t.append(time.perf_counter() - t0)
-    return sorted(t[2:])[5]
+    return min(t[2:])
 
 
 @pytest.mark.parametrize("nv", [1_000_000, 512, 1])
@@ -41,9 +41,9 @@ def test_against_the_stored_streams(life, nv):
         f, v = ints(nf), ints(nv)
     idx = life.life_build_index(ints(360), v, f, torch.ones(n, device="cuda"), 16, 360, nv, nf, precision=life.LIFE_BF16,
                                 algo=life.LIFE_ALGO_TC)
-    streams = median_s(lambda: life.life_index_export_voxel_streams(idx))
-    assert median_s(lambda: life.life_index_export(idx)) <= 1.7 * streams
-    assert median_s(lambda: life.life_index_export_tiles(idx)) <= 3.0 * streams
+    streams = best_s(lambda: life.life_index_export_voxel_streams(idx))
+    assert best_s(lambda: life.life_index_export(idx)) <= 1.7 * streams
+    assert best_s(lambda: life.life_index_export_tiles(idx)) <= 3.0 * streams
     a, voxel, _, _ = life.life_index_export(idx)
     ptr = life.life_index_export_voxel_streams(idx)[0].long()
     assert torch.equal(voxel, torch.repeat_interleave(torch.arange(nv, device="cuda", dtype=torch.int32), ptr.diff()))

@@ -49,5 +49,5 @@ def test_time_against_aligned_rows(life):
             e1.record()
             torch.cuda.synchronize()
             t.append(e0.elapsed_time(e1) * 50)
-        us[nt] = sorted(t)[3]
+        us[nt] = min(t)
     assert us[33] <= 1.7 * us[36], us
