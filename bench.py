@@ -41,11 +41,11 @@ PEAK_FALLBACK = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0}
 # hashed together); after any change to one of them the bench reports null.
 TRAFFIC_CAPTURE = {
     "src": ["spmv_tc.cu", "tile_build.cu", "tile_layout.cuh", "launch_rules.cuh", "tc_ptx.cuh", "life_internal.cuh"],
-    "sha256": "41cb72855ae39d33c93443b60d70790e1bec59391817385c4b132b8cd07d518c",
+    "sha256": "a86a1b9f3a383575754e40b77127eb71731d20cb231f95fcca5136c48fc88621",
     "nnz": 23816750,
     "bytes": {
-        "bf16-tc": {"dsc": (761856 + 0) + (197695488 + 16835328), "wc": (40148224 + 256) + (201898240 + 80384)},
-        "fp32-tc": {"dsc": (761600 + 0) + (248741632 + 19769088), "wc": (40147968 + 0) + (256169216 + 425472)},
+        "bf16-tc": {"dsc": (762112 + 0) + (197595648 + 17179136), "wc": (40147968 + 0) + (201896192 + 49920)},
+        "fp32-tc": {"dsc": (761856 + 0) + (248617984 + 19757568), "wc": (40147968 + 0) + (256477696 + 186880)},
     },
 }
 
